@@ -261,12 +261,14 @@ void prof_end(ehd_sim* s, long j) {
 // host when to stop queueing.
 int run_potential_loop(ehd_sim* s, int fixed, int max_iter) {
   if (s->resident_ok) {
+    ResidentGeom rg = s->rg;
     if (s->expire_barrier) {
       s->expire_barrier = false;
+      if (rg.cluster.size == 1) rg.cluster = ClusterGeom{};  // one CTA waits for nobody
       EHD_CUDA(launch_expire_barrier(s->b, s->stream));
     }
-    // the whole loop in one cooperative launch
-    EHD_LAUNCH(s, 1, launch_poisson_resident(s->kp, s->rg, s->rthreads, s->rsmem, s->b,
+    // the whole loop in one launch
+    EHD_LAUNCH(s, 1, launch_poisson_resident(s->kp, rg, s->rthreads, s->rsmem, s->b,
                                              s->stream));
     EHD_CUDA(cudaMemcpyAsync(s->h_ctl, s->b.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost,
                              s->stream));
@@ -605,6 +607,15 @@ int sim_create(const ehd_params* params, void* workspace, size_t workspace_bytes
           s->rg = g;
           s->rthreads = th;
           s->rsmem = sm;
+          // the library's own choice of tiles: a lattice that fits one cluster's shared
+          // memory runs its loop there (the tiles stay laid out for the diagnostics)
+          ClusterGeom cg;
+          if (depth == 0 && fixed_ty == 0)
+            for (int most = 16; most >= 8; most -= 8)
+              if (cluster_geometry(s->kp, &cg, most) && cluster_usable(s->kp, cg)) {
+                s->rg.cluster = cg;
+                break;
+              }
         }
       }
     }

@@ -310,11 +310,21 @@ struct Ctl {
   unsigned oob;             // checked build: out-of-range indices met (see EHD_IDX)
 };
 
+// Ctl::bar_count as the diagnostics set it for a solve whose waits shall run out.
+constexpr unsigned EXPIRED_BARRIER = 0x80000000u;
+
+// One-cluster potential loop (poisson_cluster.cu): `size` CTAs of at most `cap` nodes, `rows`
+// lattice rows each (size 0: not used).
+struct ClusterGeom {
+  int size, rows, cap;
+};
+
 // Tiling of the resident potential loop: ntx x nty tiles of TX x TY nodes (the last
 // column / row may be smaller), pmax perimeter slots per tile.
 struct ResidentGeom {
   int TX, TY, ntx, nty, pmax;
   int depth;  // 0: one sub-iteration per exchange; 2, 3: that many (ring and band as wide)
+  ClusterGeom cluster;  // size > 0: solves run on one cluster instead of these tiles
 };
 
 struct DevStats {
@@ -551,6 +561,16 @@ cudaError_t add_poisson_resident_node(cudaGraph_t graph, const cudaGraphNode_t* 
                                       cudaGraphNode_t* out, const KParams& kp,
                                       const ResidentGeom& g, int threads, size_t smem,
                                       const Buffers& b);
+
+// The same loop on one thread-block cluster (poisson_cluster.cu): the geometry of a lattice,
+// false if it does not fit; whether this device can launch it; the launch and its graph node.
+bool cluster_geometry(const KParams& kp, ClusterGeom* g, int max_cluster);
+bool cluster_usable(const KParams& kp, const ClusterGeom& g);
+cudaError_t launch_poisson_cluster(const KParams& kp, const ResidentGeom& rg, const Buffers& b,
+                                   cudaStream_t st);
+cudaError_t add_poisson_cluster_node(cudaGraph_t graph, const cudaGraphNode_t* deps, size_t nd,
+                                     cudaGraphNode_t* out, const KParams& kp,
+                                     const ResidentGeom& rg, const Buffers& b);
 
 cudaError_t launch_step_set(const KParams& kp, const Buffers& b, int slot, long long n,
                             int first, cudaStream_t st);

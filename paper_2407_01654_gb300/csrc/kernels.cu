@@ -924,9 +924,10 @@ __global__ void __launch_bounds__(128, HALF ? 1 : EHD_COUPLED_MIN_CTAS)
 }
 
 // Diagnostics: puts the grid barrier's arrival count half the counter range behind every
-// target, so the next on-chip solve's waits run out (bounded) instead of completing.
+// target (and tells the one-cluster loop to wait for bytes that nobody sends), so the next
+// on-chip solve's waits run out (bounded) instead of completing.
 __global__ void k_expire_barrier(Ctl* ctl) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) ctl->bar_count = 0x80000000u;
+  if (threadIdx.x == 0 && blockIdx.x == 0) ctl->bar_count = EXPIRED_BARRIER;
 }
 
 __global__ void k_stats_reset(DevStats* s) {

@@ -1815,6 +1815,7 @@ bool resident_geometry(const KParams& kp, int num_sms, ResidentGeom* g, int* thr
   g->ntx = ntx;
   g->nty = nty;
   g->depth = depth;
+  g->cluster = ClusterGeom{};
   *threads = TXR * TY / NPT;
   if (depth != 0) {
     const int D = depth, px = TXR + 2 * D;
@@ -1832,6 +1833,7 @@ bool resident_geometry(const KParams& kp, int num_sms, ResidentGeom* g, int* thr
 
 cudaError_t launch_poisson_resident(const KParams& kp, const ResidentGeom& g, int threads,
                                     size_t smem, const Buffers& b, cudaStream_t st) {
+  if (g.cluster.size > 0) return launch_poisson_cluster(kp, g, b, st);
   const void* f = resident_kernel(g.TY, g.depth, kp.scheme == 1);
   if (!f) return cudaErrorInvalidValue;
   KParams k = kp;
@@ -1849,6 +1851,7 @@ cudaError_t add_poisson_resident_node(cudaGraph_t graph, const cudaGraphNode_t* 
                                       cudaGraphNode_t* out, const KParams& kp,
                                       const ResidentGeom& g, int threads, size_t smem,
                                       const Buffers& b) {
+  if (g.cluster.size > 0) return add_poisson_cluster_node(graph, deps, nd, out, kp, g, b);
   const void* f = resident_kernel(g.TY, g.depth, kp.scheme == 1);
   if (!f) return cudaErrorInvalidValue;
   KParams k = kp;
