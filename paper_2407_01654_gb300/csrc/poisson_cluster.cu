@@ -17,21 +17,23 @@
 //   sums of sub-iteration p;
 //   collides and pushes state p + 1 into copy (p + 1) mod 3: into this CTA's shared memory,
 //   or by st.async into the neighbour's, which counts the bytes on an mbarrier there;
-//   leaves each warp's sums in a table of every CTA (st.async again);
-//   applies the rule to sub-iteration p - 1, whose sums have had a phase to arrive;
 //   meets its own CTA at a barrier.
+// Meanwhile one more warp, which owns no nodes, adds up the CTA's sums of sub-iteration p - 1,
+// sends them to every CTA's table (st.async again), waits for theirs and applies the rule; the
+// barrier hands its verdict to the others.  (With every warp sending its own sums and deciding
+// for itself the rule cost 0.4 to 0.5 us of a sub-iteration, as much as the rest of it.)
 // A phase starts once the neighbours' rows are counted in.  There is no cluster-wide barrier:
 // its release waits for every outstanding remote store (a memory barrier, 38 % of a phase when
 // this loop used barrier.cluster: 1.44 us per sub-iteration at 128 x 128), while a counted
-// store needs none.  CTAs drift by at most one phase from a neighbour (it needs our rows) and
-// two from any other (the rule needs every CTA's sums), so two row barriers, four table slots
-// and, because all take the same decision before they push on, three copies are enough; state
-// p - 1 stays in its copy until the rule has judged it.  With two copies (lattices that leave
+// store needs none.  CTAs drift by at most one phase (a neighbour needs our rows, and the rule
+// every CTA's sums), so two row barriers, two table slots and, because all take the same
+// decision before they go on, three copies are enough; state p - 1 stays in its copy until the
+// rule has judged it.  With two copies (lattices that leave
 // no room for three) the rule is applied before the push.  A fixed count needs no rule: only
 // its last phase, which finds the final state in its registers, forms sums.
 //
 // A population that would cross a wall returns to its own node by the anti-bounce-back rule,
-// written by the node itself.  Sums are FP32 throughout in a fixed order; every warp adds the
+// written by the node itself.  Sums are FP32 throughout in a fixed order; every CTA adds the
 // same table in the same order and takes the same decision.  The order is not the tiled
 // loop's, whose sums can differ from these in the last bits; where that could matter, with
 // num within 2e-5 of tol^2 den (both orders are far closer than that to the exact sums: at
@@ -133,13 +135,11 @@ struct ClusterShape {
   static_assert(NPT % 2 == 0 && CAP % (32 * NPT) == 0, "whole warps of packed pairs");
   static constexpr int THREADS = CAP / NPT;
   static constexpr int WARPS = THREADS / 32;
+  static constexpr int LAUNCH = THREADS + 32;  // and the warp that keeps the sums
   static constexpr int COPIES = CAP <= 2048 ? 3 : 2;
   static constexpr bool KEEP = NPT <= 2 || THREADS <= 384;  // push addresses kept in registers
   static constexpr int COPY = 8 * CAP;  // floats of one copy
-  static constexpr int SLOTS = 4;         // table slots, one per phase in turn
-  static constexpr int ENTRIES = MAX_CLUSTER * WARPS;  // table entries (pairs of sums) a slot
-  static_assert(ENTRIES % 64 == 0, "read as whole float4 by a warp");
-  static constexpr size_t SMEM = sizeof(float) * (size_t)COPIES * COPY + sizeof(float2) * SLOTS * ENTRIES;
+  static constexpr size_t SMEM = sizeof(float) * (size_t)COPIES * COPY;
 };
 
 template <int V>
@@ -153,15 +153,17 @@ __device__ __forceinline__ void each_direction(F f) {
 }  // namespace
 
 template <int CAP, int NPT, bool CONV>
-__global__ void __launch_bounds__(CAP / NPT, 1)
+__global__ void __launch_bounds__(ClusterShape<CAP, NPT>::LAUNCH, 1)
     k_poisson_cluster(KParams k, int rows, ResidentGeom rg, float* __restrict__ hbuf,
                       const float2* __restrict__ aq, float2* __restrict__ scratch, Ctl* ctl) {
   using S = ClusterShape<CAP, NPT>;
   constexpr int NP = NPT / 2;
   constexpr int T = S::THREADS;
-  __shared__ __align__(8) unsigned long long s_rows[2], s_sums[S::SLOTS];  // mbarriers
-  extern __shared__ __align__(16) float smc[];  // [COPIES][8][CAP], then the table
-  float2* table = reinterpret_cast<float2*>(smc + S::COPIES * S::COPY);  // [SLOTS][ENTRIES]
+  __shared__ __align__(8) unsigned long long s_rows[2], s_sums[2];  // mbarriers
+  __shared__ __align__(8) float2 s_table[2][MAX_CLUSTER];  // every CTA's sums, in turn
+  __shared__ float2 s_warp[2][S::WARPS];                   // this CTA's warps' sums, in turn
+  __shared__ int s_verdict;
+  extern __shared__ __align__(16) float smc[];  // [COPIES][8][CAP]
 
   const int nx = k.nx, ny = k.ny;
   const size_t N = (size_t)k.N;
@@ -170,6 +172,7 @@ __global__ void __launch_bounds__(CAP / NPT, 1)
   const int th = min(rows, ny - row0);
   const int nloc = th * nx;
   const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const bool keeper = warp == S::WARPS;  // the warp that keeps the sums
   const int parity = __ldg(&ctl->parity);
   float* __restrict__ hsrc = hbuf + (size_t)parity * NH * N;
   const int g0 = row0 * nx;  // my first node
@@ -180,7 +183,7 @@ __global__ void __launch_bounds__(CAP / NPT, 1)
   bool valid[NPT];
 #pragma unroll
   for (int s = 0; s < NPT; ++s) {
-    valid[s] = tid + s * T < nloc;
+    valid[s] = !keeper && tid + s * T < nloc;
     const size_t g = EHD_IDX(k, g0 + (valid[s] ? tid + s * T : 0), N);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
@@ -275,19 +278,19 @@ __global__ void __launch_bounds__(CAP / NPT, 1)
     }
   }
   float *own0 = smc + tid, *up0 = own0 + nx, *dn0 = own0 - nx;
-  // where this warp's sums go: lane c writes CTA c's table
+  // where the CTA's sums go: lane c writes CTA c's table
   const unsigned to = (unsigned)(lane < C ? lane : 0);
-  const unsigned my_table =
-      (C > 1 ? map_rank(smem_addr(table), to) : smem_addr(table)) + 8u * (unsigned)(rank * S::WARPS + warp);
-  const unsigned sums_bar = C > 1 ? map_rank(smem_addr(s_sums), to) : 0u;
+  const unsigned my_table = map_rank(smem_addr(s_table), to) + 8u * (unsigned)rank;
+  const unsigned sums_bar = map_rank(smem_addr(s_sums), to);
   const unsigned my_rows = smem_addr(s_rows), my_sums = smem_addr(s_sums);
-  // table entries past the cluster's warps stay zero
-  for (int j = tid; j < S::SLOTS * S::ENTRIES; j += T) table[j] = make_float2(0.0f, 0.0f);
+  if (tid < 2 * MAX_CLUSTER) s_table[0][tid] = make_float2(0.0f, 0.0f);  // past C: zero
   // no remote store before every CTA of the cluster has started and set up its barriers
   if (C > 1) {
     if (tid == 0) {
-      for (int j = 0; j < 2; ++j) mbar_init(my_rows + 8u * j);
-      for (int j = 0; j < S::SLOTS; ++j) mbar_init(my_sums + 8u * j);
+      for (int j = 0; j < 2; ++j) {
+        mbar_init(my_rows + 8u * j);
+        mbar_init(my_sums + 8u * j);
+      }
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     cluster_arrive();
@@ -297,16 +300,14 @@ __global__ void __launch_bounds__(CAP / NPT, 1)
   }
 
   float2 vold[NP];          // varphi of the state in the registers
-  float2 dnow[NP];          // its change from the state before
-  float2 v1[NP];            // and the potential it changed from
-  float2 d1[NP], v2[NP];    // the same two one sub-iteration earlier
+  float2 v1[NP], v2[NP];    // and of the two states before it
   float rel = 0.0f;
   int conv = 0, it = 0;
   bool fail = false;  // a wait of this thread ran out
 
   // The parity of the sums' barrier at phase p: under the rule slots take turns from phase 1
   // on; a fixed count uses one of them, once.
-  auto sums_parity = [&](int p) { return fixed > 0 ? 0u : (unsigned)((p - 1) / S::SLOTS) & 1u; };
+  auto sums_parity = [&](int p) { return fixed > 0 ? 0u : (unsigned)((p - 1) >> 1) & 1u; };
   auto meet = [&]() {  // every thread of the cluster, global memory included
     if (C > 1) {
       __syncwarp();
@@ -316,22 +317,34 @@ __global__ void __launch_bounds__(CAP / NPT, 1)
       __syncthreads();
     }
   };
-  // The stopping sums of the previous sub-iteration (its changes d1 from the potentials v2), in
-  // the order of the one-step tiled loop: per thread of a 64 x TY tile the nodes of one column TY / 4 rows
-  // apart, then lanes, warps and tiles.  Every node leaves its change and its old potential in
-  // scratch; the cluster's warps share out the tiles' warps.
-  auto tiled_sums = [&](float& sa, float& sb) {
+  // The potential of the state after sub-iteration st, and its change from potential v as the
+  // one-step tiled loop forms it: from the rounded new potential in odd sub-iterations (its own
+  // layout), with one rounding in even ones.
+  auto change = [&](int st, const float2 (&hn)[8], float2 v, float2& vnew) -> float2 {
+    const float2 hsum = h_sum8x2(hn);
+    // (scalar products: a packed one may be contracted with the addition)
+    vnew = make_float2(h_varphi(hsum.x), h_varphi(hsum.y));
+    return (st & 1) ? __fadd2_rn(vnew, neg2(v)) : __ffma2_rn(hsum, f2(9.0f / 5.0f), neg2(v));
+  };
+  // The stopping sums of sub-iteration st, whose state is in h and which began from potential
+  // v, in the order of the one-step tiled loop: per thread of a 64 x TY tile the nodes of one
+  // column TY / 4 rows apart, then lanes, warps and tiles.  Every node leaves its change and
+  // its old potential in scratch; the cluster's warps share out the tiles' warps.
+  auto tiled_sums = [&](int st, float& sa, float& sb, const float2 (&v)[NP]) {
+    float2 d[NP], vn;
+#pragma unroll
+    for (int j = 0; j < NP; ++j) d[j] = change(st, h[j], v[j], vn);
 #pragma unroll
     for (int s = 0; s < NPT; ++s) {
       if (valid[s])
-        scratch[g0 + tid + s * T] = (s & 1) ? make_float2(d1[s >> 1].y, v2[s >> 1].y)
-                                            : make_float2(d1[s >> 1].x, v2[s >> 1].x);
+        scratch[g0 + tid + s * T] = (s & 1) ? make_float2(d[s >> 1].y, v[s >> 1].y)
+                                            : make_float2(d[s >> 1].x, v[s >> 1].x);
     }
     meet();
     const int nw = rg.TY / 2, step = rg.TY / 4, tiles = rg.ntx * rg.nty;
     float2* wsum = scratch + N;
-    for (int v = rank * S::WARPS + warp; v < tiles * nw; v += C * S::WARPS) {
-      const int t = v / nw, w = v - t * nw;
+    for (int u = keeper ? tiles * nw : rank * S::WARPS + warp; u < tiles * nw; u += C * S::WARPS) {
+      const int t = u / nw, w = u - t * nw;
       const int x = (t % rg.ntx) * 64 + (w & 1) * 32 + lane, y0 = (t / rg.ntx) * rg.TY;
       float num = 0.0f, den = 0.0f;
 #pragma unroll
@@ -345,7 +358,7 @@ __global__ void __launch_bounds__(CAP / NPT, 1)
       }
       const float part = warp_sum2(num, den, lane);
       const float other = __shfl_xor_sync(0xffffffffu, part, 16);
-      if (lane == 0) __stcg(wsum + v, make_float2(part, other));
+      if (lane == 0) __stcg(wsum + u, make_float2(part, other));
     }
     meet();
     float a = 0.0f, b = 0.0f;
@@ -364,50 +377,62 @@ __global__ void __launch_bounds__(CAP / NPT, 1)
     sb = lane < 16 ? other : part;
     meet();  // scratch may be written again
   };
-  // The stopping rule for sub-iteration st, from the sums that every warp of every CTA left
-  // in its table slot.
-  auto decide = [&](int st) -> bool {
-    const int slot = st & (S::SLOTS - 1);
-    if (C > 1 && !mbar_wait(my_sums + 8u * slot, sums_parity(st))) fail = true;
-    const float2* e = table + slot * S::ENTRIES;
-    const float4* e4 = reinterpret_cast<const float4*>(e);
-    float4 v = e4[lane];
-    if constexpr (S::ENTRIES > 64) {
-      const int n = C * S::WARPS;  // entries in use; the rest hold zero
-      for (int j = 32; 2 * j < n; j += 32) {
-        const float4 w = e4[lane + j];
-        v.x += w.x;
-        v.y += w.y;
-        v.z += w.z;
-        v.w += w.w;
-      }
-    }
-    const float part = warp_sum2(v.x + v.z, v.y + v.w, lane);
+  // The keeper adds up the CTA's sums of sub-iteration st (after the CTA barrier that followed
+  // them) and sends them to every CTA.
+  auto send_sums = [&](int st) {
+    if (C == 1) return;
+    const float2 v = lane < S::WARPS ? s_warp[st & 1][lane] : make_float2(0.0f, 0.0f);
+    const float part = warp_sum2(v.x, v.y, lane);
     const float other = __shfl_xor_sync(0xffffffffu, part, 16);
-    float sa = lane < 16 ? part : other, sb = lane < 16 ? other : part;
-    auto ratio = [&](float n, float d) {
-      return n == 0.0f && d == 0.0f ? 0.0f : (d == 0.0f ? __int_as_float(0x7f800000) : sqrtf(n / d));
-    };
-    conv = 1;
-    if (fixed == 0) {
-      if (tol_ok && sb > 1e-25f && sb < 1e25f && sa > 1.00002f * tol2 * sb) {
+    if (lane == 0) mbar_expect(my_sums + 8u * (unsigned)(st & 1), 8u * (unsigned)C);
+    if (lane < C && !fail)
+      st_async2(my_table + 8u * MAX_CLUSTER * (unsigned)(st & 1), lane < 16 ? part : other,
+                lane < 16 ? other : part, sums_bar + 8u * (unsigned)(st & 1));
+  };
+  // The sums of sub-iteration st over the lattice, from the CTAs' (with one CTA, its warps').
+  auto all_sums = [&](int st, float& sa, float& sb) {
+    const float2* e = C > 1 ? s_table[st & 1] : s_warp[st & 1];
+    const int n = C > 1 ? C : S::WARPS;
+    if (C > 1 && !mbar_wait(my_sums + 8u * (unsigned)(st & 1), sums_parity(st))) fail = true;
+    float part = 0.0f;  // the low lanes add num, the high lanes den
+    for (int j = lane & 15; j < n; j += 16) part += reinterpret_cast<const float*>(e + j)[lane >> 4];
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+    const float other = __shfl_xor_sync(0xffffffffu, part, 16);
+    sa = lane < 16 ? part : other;
+    sb = lane < 16 ? other : part;
+  };
+  auto ratio = [&](float n, float d) {
+    return n == 0.0f && d == 0.0f ? 0.0f : (d == 0.0f ? __int_as_float(0x7f800000) : sqrtf(n / d));
+  };
+  // The stopping rule for sub-iteration st from its sums: GO_ON, STOP (it, rel and conv set) or
+  // UNSURE, which wants the sums in the tiled loop's order (sure = true takes them as such).
+  enum { GO_ON = 0, STOP = 1, UNSURE = 2 };
+  auto decide = [&](int st, float sa, float sb, bool sure) -> int {
+    if (fixed > 0) {
+      conv = 1;
+    } else {
+      const bool plain = !sure && tol_ok && sb > 1e-25f && sb < 1e25f;
+      if (plain && sa > 1.00002f * tol2 * sb) {
         conv = 0;
-      } else if (tol_ok && sb > 1e-25f && sb < 1e25f && sa < 0.99998f * tol2 * sb) {
+      } else if (plain && sa < 0.99998f * tol2 * sb) {
         conv = st >= min_iter;
       } else if (st < min_iter && st < max_iter) {
         conv = 0;  // whatever the sums say
+      } else if (!sure && sb != 0.0f) {  // all zero is zero in any order
+        return UNSURE;
       } else {
-        if (!(sb == 0.0f)) tiled_sums(sa, sb);  // all zero is zero in any order
         conv = (st >= min_iter) && ((double)ratio(sa, sb) < tol);
       }
-      if (!conv && st < max_iter) return false;
+      if (!conv && st < max_iter) return GO_ON;
     }
     rel = ratio(sa, sb);
     it = st;
-    return true;
+    return STOP;
   };
   auto load_state = [&](auto copy) {
     constexpr int at = decltype(copy)::value * S::COPY;
+    if (keeper) return;  // owns no nodes: its cells would lie past the copies
 #pragma unroll
     for (int j = 0; j < NP; ++j)
 #pragma unroll
@@ -508,81 +533,99 @@ __global__ void __launch_bounds__(CAP / NPT, 1)
   // ran out.
   auto phase = [&](int p, auto RD, auto WR, auto OLD) -> int {
     const bool last = fixed > 0 && p == fixed;
-    const bool sums = fixed == 0 || last;
-    const int slot = p & (S::SLOTS - 1);
-    if (C > 1) {
-      if (tid == 0) {  // what this phase's neighbours and all CTAs' warps will send
-        if (!last) mbar_expect(my_rows + 8u * (unsigned)(p & 1), row_bytes);
-        if (sums) mbar_expect(my_sums + 8u * (unsigned)slot, 8u * (unsigned)(C * S::WARPS));
-      }
+    const bool rule = fixed == 0 && p > 1;
+    int verdict = GO_ON;
+    bool pushed = !last;
+    float sa, sb;
+    if (keeper) {
+      // what this phase's neighbours will send
+      if (C > 1 && lane == 0 && !last) mbar_expect(my_rows + 8u * (unsigned)(p & 1), row_bytes);
+      if (rule) send_sums(p - 1);
+    } else {
       // the neighbours' rows of state p, pushed in their phase p - 1
-      if (!mbar_wait(my_rows + 8u * (unsigned)((p - 1) & 1), (unsigned)((p - 1) >> 1) & 1u)) fail = true;
+      if (C > 1 && !mbar_wait(my_rows + 8u * (unsigned)((p - 1) & 1), (unsigned)((p - 1) >> 1) & 1u))
+        fail = true;
+      load_state(RD);
     }
-    load_state(RD);
-    float num = 0.0f, den = 0.0f;
+    if (S::COPIES == 2 && rule) {
+      // no copy to spare: every warp decides before the push
+      all_sums(p - 1, sa, sb);
+      verdict = decide(p - 1, sa, sb, false);
+      if (verdict == UNSURE) {
+        load_state(OLD);
+        tiled_sums(p - 1, sa, sb, v1);
+        verdict = decide(p - 1, sa, sb, true);
+        load_state(RD);
+      }
+      pushed = verdict == GO_ON;
+    }
+    if (!keeper) {
+      float num = 0.0f, den = 0.0f;
 #pragma unroll
-    for (int j = 0; j < NP; ++j) {
-      // the change of the potential as the one-step tiled loop forms it: from the rounded new
-      // potential in odd sub-iterations (its own layout), with one rounding in even ones
-      const float2 hsum = h_sum8x2(h[j]);
-      float2 vnew = h_varphi2(hsum);
-      asm volatile("" : "+f"(vnew.x), "+f"(vnew.y));  // keeps the product's rounding
-      const float2 d = (p & 1) ? __fadd2_rn(vnew, neg2(vold[j]))
-                               : __ffma2_rn(hsum, f2(9.0f / 5.0f), neg2(vold[j]));
-      d1[j] = dnow[j];
-      v2[j] = v1[j];
-      v1[j] = vold[j];
-      dnow[j] = d;
-      if (valid[2 * j]) {
-        num = __fmaf_rn(d.x, d.x, num);
-        den = __fmaf_rn(vold[j].x, vold[j].x, den);
+      for (int j = 0; j < NP; ++j) {
+        float2 vnew;
+        const float2 d = change(p, h[j], vold[j], vnew);
+        if (S::COPIES == 3) v2[j] = v1[j];
+        v1[j] = vold[j];
+        if (valid[2 * j]) {
+          num = __fmaf_rn(d.x, d.x, num);
+          den = __fmaf_rn(vold[j].x, vold[j].x, den);
+        }
+        if (valid[2 * j + 1]) {
+          num = __fmaf_rn(d.y, d.y, num);
+          den = __fmaf_rn(vold[j].y, vold[j].y, den);
+        }
+        vold[j] = vnew;
       }
-      if (valid[2 * j + 1]) {
-        num = __fmaf_rn(d.y, d.y, num);
-        den = __fmaf_rn(vold[j].y, vold[j].y, den);
+      if (pushed && !fail) collide_push(p, WR);
+      if (fixed == 0 || last) {
+        const float part = warp_sum2(num, den, lane);
+        const float other = __shfl_xor_sync(0xffffffffu, part, 16);
+        if (lane == 0) s_warp[p & 1][warp] = make_float2(part, other);
       }
-      vold[j] = vnew;
+    } else if (S::COPIES == 3 && rule) {
+      all_sums(p - 1, sa, sb);
+      verdict = decide(p - 1, sa, sb, false);
+      if (verdict != GO_ON && lane == 0) s_verdict = verdict;
     }
-    bool done = false;
-    if (S::COPIES == 2 && p > 1 && fixed == 0) done = decide(p - 1);
-    const bool push = !last && !(S::COPIES == 2 && done);
-    if (push && !fail) collide_push(p, WR);
-    if (sums && !fail) {
-      const float part = warp_sum2(num, den, lane);
-      const float other = __shfl_xor_sync(0xffffffffu, part, 16);
-      const float sn = lane < 16 ? part : other, sd = lane < 16 ? other : part;
-      const unsigned at = my_table + 8u * (unsigned)(slot * S::ENTRIES);
-      if (C > 1) {
-        if (lane < C) st_async2(at, sn, sd, sums_bar + 8u * (unsigned)slot);
-      } else if (lane == 0) {
-        asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(at), "f"(sn), "f"(sd) : "memory");
+    if (__syncthreads_or(fail || verdict != GO_ON)) {
+      if (__syncthreads_or(fail)) return 2;
+      if (S::COPIES == 3) {
+        verdict = s_verdict;
+        if (verdict == UNSURE) {
+          load_state(OLD);
+          tiled_sums(p - 1, sa, sb, v2);
+          verdict = decide(p - 1, sa, sb, true);
+          if (verdict == GO_ON) return 0;
+        }
       }
-    }
-    if (S::COPIES == 3 && p > 1 && fixed == 0) done = decide(p - 1);
-    if (__syncthreads_or(fail)) return 2;
-    if (last) {
-      decide(p);  // the fixed count's state is in the registers
+      if (!keeper) {
+        load_state(OLD);
+        // what the neighbours sent before they took the same decision must have arrived before
+        // this CTA leaves
+        if (C > 1 && pushed && !mbar_wait(my_rows + 8u * (unsigned)(p & 1), (unsigned)(p >> 1) & 1u))
+          fail = true;
+      }
       return __syncthreads_or(fail) ? 2 : 1;
     }
-    if (!done) return 0;
-    load_state(OLD);
-    if (C > 1) {
-      // whatever the others sent before they took the same decision must have arrived before
-      // this CTA leaves
-      if (push && !mbar_wait(my_rows + 8u * (unsigned)(p & 1), (unsigned)(p >> 1) & 1u)) fail = true;
-      if (!mbar_wait(my_sums + 8u * (unsigned)slot, sums_parity(p))) fail = true;
+    if (last) {  // the fixed count's state is in the registers
+      if (keeper) {
+        send_sums(p);
+        all_sums(p, sa, sb);
+        decide(p, sa, sb, false);
+      }
+      return __syncthreads_or(fail) ? 2 : 1;
     }
-    return __syncthreads_or(fail) ? 2 : 1;
+    return 0;
   };
 
   // phase 0: the state is in the registers
 #pragma unroll
   for (int j = 0; j < NP; ++j) {
     v1[j] = v2[j] = vold[j] = h_varphi2(h_sum8x2(h[j]));
-    dnow[j] = d1[j] = f2(0.0f);
   }
-  if (C > 1 && tid == 0) mbar_expect(my_rows, row_bytes);
-  collide_push(0, Const<1>{});
+  if (C > 1 && keeper && lane == 0) mbar_expect(my_rows, row_bytes);
+  if (!keeper) collide_push(0, Const<1>{});
   __syncthreads();
   int end = 0;
   if constexpr (S::COPIES == 3) {
@@ -614,7 +657,7 @@ __global__ void __launch_bounds__(CAP / NPT, 1)
 #pragma unroll
     for (int i = 0; i < 8; ++i) hsrc[i * N + g] = (s & 1) ? h[s >> 1][i].y : h[s >> 1][i].x;
   }
-  if (rank == 0 && tid == 0) {
+  if (rank == 0 && keeper && lane == 0) {
     ctl->iter = it;
     ctl->rel = (double)rel;
     ctl->converged = conv;
@@ -632,15 +675,15 @@ struct ClusterKernel {
 template <int CAP, int NPT>
 ClusterKernel cluster_kernel_of() {
   using S = ClusterShape<CAP, NPT>;
-  return {CAP, S::THREADS, S::SMEM,
+  return {CAP, S::LAUNCH, S::SMEM,
           {(const void*)k_poisson_cluster<CAP, NPT, false>,
            (const void*)k_poisson_cluster<CAP, NPT, true>}};
 }
 const ClusterKernel* cluster_kernels(int* n) {
   static const ClusterKernel all[] = {
       cluster_kernel_of<256, 2>(),  cluster_kernel_of<512, 2>(),  cluster_kernel_of<768, 2>(),
-      cluster_kernel_of<1024, 2>(), cluster_kernel_of<1536, 4>(), cluster_kernel_of<2048, 4>(),
-      cluster_kernel_of<2560, 4>(), cluster_kernel_of<3072, 6>()};
+      cluster_kernel_of<1024, 2>(), cluster_kernel_of<1408, 4>(), cluster_kernel_of<1920, 4>(),
+      cluster_kernel_of<2432, 4>(), cluster_kernel_of<2880, 6>()};
   *n = (int)(sizeof(all) / sizeof(all[0]));
   return all;
 }
@@ -726,7 +769,7 @@ bool cluster_usable(const KParams& kp, const ClusterGeom& g) {
 // moments pass's partials, which the coupled pass still reads, are at most N / 256 at the
 // start of the lower half).
 static float2* cluster_scratch(const Buffers& b) {
-  static_assert(MAX_CLUSTER * 3072 + 256 * 32 <= MAX_PARTIALS, "nodes and warps of all tiles");
+  static_assert(MAX_CLUSTER * 2880 + 256 * 32 <= MAX_PARTIALS, "nodes and warps of all tiles");
   return reinterpret_cast<float2*>(b.partials + MAX_PARTIALS / 2);
 }
 

@@ -11,11 +11,20 @@ from paper_2407_01654_gb300 import workloads as wl
 
 pytestmark = pytest.mark.gpu
 
-# nx, ny: CTAs x rows x capacity are (1, 32, 512), (3, 7, 256), (1, 7, 256), (16, 38, 256),
-# (9, 1, 512), (16, 4, 256), (16, 8, 1024), (15, 7, 1536), (15, 10, 2048), (15, 13, 2560),
-# (16, 16, 3072), then one beyond
-SHAPES = [(16, 32), (27, 19), (3, 7), (1, 600), (300, 9), (64, 64), (128, 128), (200, 100),
-          (180, 149), (190, 194), (192, 256), (193, 256)]
+# nx, ny (CTAs, rows of each, capacity): one CTA, its largest and beyond; single rows and
+# columns; every capacity, full and ragged; the largest that fits and one beyond
+SHAPES = [(16, 32),    # 1, 32, 512
+          (27, 19),    # 3, 7, 256
+          (3, 7),      # 1, 7, 256
+          (1, 600),    # 3, 200, 256
+          (300, 9),    # 5, 2, 768
+          (64, 64),    # 16, 4, 256
+          (128, 128),  # 16, 8, 1024
+          (200, 100),  # 15, 7, 1408
+          (180, 149),  # 15, 10, 1920
+          (187, 194),  # 15, 13, 2432
+          (180, 256),  # 16, 16, 2880
+          (181, 256)]  # tiled
 
 
 @pytest.fixture(scope="module")
@@ -84,7 +93,7 @@ def test_rule_stops_where_the_tiled_loop_stops(gpu, nx, ny):
 
 @pytest.mark.parametrize("k", [40, 41])
 @pytest.mark.parametrize("nx,ny,walls,scheme", [(4, 64, 1, 0), (64, 64, 0, 0), (64, 64, 1, 1),
-                                                (200, 100, 1, 0), (192, 256, 1, 0),
+                                                (200, 100, 1, 0), (180, 256, 1, 0),
                                                 (60, 7, 1, 0), (64, 24, 1, 0), (100, 40, 0, 0),
                                                 (128, 60, 1, 0)])
 def test_rule_on_the_last_bit(gpu, nx, ny, walls, scheme, k):
