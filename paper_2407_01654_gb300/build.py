@@ -23,7 +23,7 @@ BUILD_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libehd.so")
 LIB_CHECKED = os.path.join(HERE, "libehd_checked.so")
 SOURCES = ["kernels.cu", "poisson.cu", "poisson_resident.cu", "poisson_cluster.cu",
-           "noalloc.cu", "batch.cu", "api.cu", "diag.cu", "slabs.cu"]
+           "poisson_multi.cu", "noalloc.cu", "batch.cu", "api.cu", "diag.cu", "slabs.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "--expt-relaxed-constexpr", "-I", os.path.join(ROOT, "include")]

@@ -278,17 +278,23 @@ int run_potential_loop(ehd_sim* s, int fixed, int max_iter) {
     s->last_k = s->h_ctl->iter;
     return s->h_ctl->converged ? EHD_OK : EHD_ERR_NOT_CONVERGED;
   }
+  const bool multi = multi_ok(s->kp);
+  auto launch = [&]() {
+    return multi ? launch_poisson_multi(s->kp, s->b, s->stream) : launch_poisson(s->kp, s->b, s->stream);
+  };
   if (fixed > 0) {
-    for (int i = 0; i < fixed; ++i) EHD_LAUNCH(s, 1, launch_poisson(s->kp, s->b, s->stream));
+    const int n = multi ? multi_launches(fixed) : fixed;
+    for (int i = 0; i < n; ++i) EHD_LAUNCH(s, 1, launch());
     return EHD_OK;
   }
   int queued = 0;
-  int chunk = s->last_k + 1;
+  // (several sub-iterations a launch: the last solve's launches, and one that repeats)
+  int chunk = multi ? multi_launches(s->last_k) + 1 : s->last_k + 1;
   const size_t first_pair = s->ev_used;
   for (;;) {
     if (chunk > max_iter - queued + 1) chunk = max_iter - queued + 1;
     if (chunk < 1) chunk = 1;
-    for (int i = 0; i < chunk; ++i) EHD_LAUNCH(s, 1, launch_poisson(s->kp, s->b, s->stream));
+    for (int i = 0; i < chunk; ++i) EHD_LAUNCH(s, 1, launch());
     queued += chunk;
     EHD_CUDA(cudaMemcpyAsync(s->h_ctl, s->b.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost,
                              s->stream));
@@ -297,7 +303,8 @@ int run_potential_loop(ehd_sim* s, int fixed, int max_iter) {
       s->last_k = s->h_ctl->iter;
       // launches after the loop finished did no work: file them under their own kind
       if (s->profiling && s->ev_used >= first_pair)
-        for (size_t j = first_pair + (size_t)s->h_ctl->iter; j < s->ev_used; ++j)
+        for (size_t j = first_pair + (size_t)(multi ? s->h_ctl->plaunch : s->h_ctl->iter);
+             j < s->ev_used; ++j)
           s->ev_kind[j] = 2;
       return s->h_ctl->converged ? EHD_OK : EHD_ERR_NOT_CONVERGED;
     }
@@ -627,6 +634,11 @@ int sim_create(const ehd_params* params, void* workspace, size_t workspace_bytes
       return EHD_ERR_INVALID_ARG;  // the lattice does not fit on chip on this device
     }
   }
+  if (!s->resident_ok && multi_ok(s->kp) && multi_prepare(s->kp) != cudaSuccess) {
+    cudaGetLastError();
+    ehd_destroy(s);
+    return EHD_ERR_CUDA;
+  }
   if (cudaMallocHost(&s->h_ctl, sizeof(Ctl)) != cudaSuccess ||
       cudaMallocHost(&s->h_stats, sizeof(DevStats)) != cudaSuccess ||
       cudaMallocHost(&s->h_stage, sizeof(float) * NIO * (size_t)N) != cudaSuccess) {
@@ -778,6 +790,8 @@ static int fill_stats(ehd_sim* s, ehd_stats* out) {
   out->kernel_launches = s->launches + 2LL * s->graph_steps;
   if (s->resident_ok)
     out->kernel_launches += s->graph_steps;
+  else if (multi_ok(s->kp))
+    out->kernel_launches += (int64_t)d.plaunches - s->host_iters;
   else
     out->kernel_launches += (int64_t)d.iters_total - s->host_iters;
   int status = EHD_OK;
@@ -849,7 +863,7 @@ int ehd_step(ehd_sim* s, int nsteps, ehd_stats* out) {
       }
       if (st == EHD_ERR_CUDA || st == EHD_ERR_TIMEOUT) return st;
       if (st != EHD_OK) status = st;
-      if (!s->resident_ok) s->host_iters += s->h_ctl->iter;
+      if (!s->resident_ok) s->host_iters += multi_ok(s->kp) ? s->h_ctl->plaunch : s->h_ctl->iter;
       NvtxRange r("coupled");
       EHD_LAUNCH(s, 3, launch_coupled(s->kp, s->b, s->cur, s->stream));
     }

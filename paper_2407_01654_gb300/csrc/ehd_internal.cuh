@@ -307,6 +307,9 @@ struct Ctl {
   double slab_num, slab_den;// one slab's stopping sums of its last sub-iteration
   int mpart_n;              // > 0: the moments pass left its FP64 sums as this many
                             // per-CTA partials, reduced by the coupled pass
+  int redo;                 // streaming, several sub-iterations a launch: > 0: the rule stopped
+                            // the loop inside the last launch; the next one repeats that many
+  int plaunch;              // and its launches in the current solve
   unsigned oob;             // checked build: out-of-range indices met (see EHD_IDX)
 };
 
@@ -329,7 +332,8 @@ struct ResidentGeom {
 
 struct DevStats {
   int iters_total, iters_min, iters_max, not_converged, nonfinite, steps;
-  int barrier_error, pad;
+  int barrier_error;
+  int plaunches;            // streaming launches, where a launch makes several sub-iterations
   double last_rel, sum_phi, sum_q;
 };
 
@@ -561,6 +565,16 @@ cudaError_t add_poisson_resident_node(cudaGraph_t graph, const cudaGraphNode_t* 
                                       cudaGraphNode_t* out, const KParams& kp,
                                       const ResidentGeom& g, int threads, size_t smem,
                                       const Buffers& b);
+
+// Streaming with several sub-iterations per launch (poisson_multi.cu).
+constexpr long long MULTI_MIN_NODES = 600000;
+bool multi_ok(const KParams& kp);
+cudaError_t multi_prepare(const KParams& kp);
+int multi_launches(int fixed);  // launches of a fixed count
+cudaError_t launch_poisson_multi(const KParams& kp, const Buffers& b, cudaStream_t st);
+cudaError_t add_poisson_multi_node(cudaGraph_t g, const cudaGraphNode_t* deps, size_t nd,
+                                   cudaGraphNode_t* out, const KParams& kp, const Buffers& b,
+                                   const cudaGraphConditionalHandle* handle);
 
 // The same loop on one thread-block cluster (poisson_cluster.cu): the geometry of a lattice,
 // false if it does not fit; whether this device can launch it; the launch and its graph node.

@@ -332,6 +332,8 @@ __device__ __forceinline__ void moments_tail(const KParams& k, const StepState* 
     ctl->ticket_m = 0u;
     ctl->bar_count = 0u;
     ctl->mpart_n = 0;
+    ctl->redo = 0;
+    ctl->plaunch = 0;
     __threadfence();
   }
 }
@@ -379,6 +381,8 @@ __device__ __forceinline__ void moments_partial_only(const KParams& k,
     ctl->ticket_m = 0u;
     ctl->bar_count = 0u;
     ctl->mpart_n = nblk;
+    ctl->redo = 0;
+    ctl->plaunch = 0;
   }
 }
 
@@ -555,6 +559,7 @@ __device__ __forceinline__ void coupled_record(const KParams& k, StepState* ss, 
   stats->sum_phi = ld_cg(&ctl->sum_phi);
   stats->sum_q = ld_cg(&ctl->sum_q);
   stats->barrier_error |= ld_cg(&ctl->bar_error);
+  stats->plaunches += ld_cg(&ctl->plaunch);
   stats->steps += 1;
 }
 
@@ -938,6 +943,7 @@ __global__ void k_stats_reset(DevStats* s) {
   s->nonfinite = 0;
   s->steps = 0;
   s->barrier_error = 0;
+  s->plaunches = 0;
   s->last_rel = 0.0;
   s->sum_phi = 0.0;
   s->sum_q = 0.0;
@@ -1316,6 +1322,14 @@ cudaError_t build_step_graph(const KParams& kp, const Buffers& b, int cur, doubl
           cudaSuccess)
         return done(e);
       last = pn;
+    } else if (multi_ok(kp) && fixed_iter > 0 && multi_launches(fixed_iter) <= 8) {
+      // a fixed count's few launches in a row, without a condition between them (after a
+      // non-finite field the first one ends the loop and the others return at once)
+      for (int l = 0; l < multi_launches(fixed_iter); ++l) {
+        if ((e = add_poisson_multi_node(g, &last, 1, &pn, kp, b, nullptr)) != cudaSuccess)
+          return done(e);
+        last = pn;
+      }
     } else {
       // each step's WHILE node has its own handle, reset to 1 at every launch of the graph
       cudaGraphConditionalHandle h;
@@ -1328,7 +1342,9 @@ cudaError_t build_step_graph(const KParams& kp, const Buffers& b, int cur, doubl
       cp.conditional.type = cudaGraphCondTypeWhile;
       cp.conditional.size = 1;
       if ((e = cudaGraphAddNode(&wn, g, &last, nullptr, 1, &cp)) != cudaSuccess ||
-          (e = add_poisson_node(cp.conditional.phGraph_out[0], &pn, kp, b, h)) != cudaSuccess)
+          (e = multi_ok(kp)
+                   ? add_poisson_multi_node(cp.conditional.phGraph_out[0], nullptr, 0, &pn, kp, b, &h)
+                   : add_poisson_node(cp.conditional.phGraph_out[0], &pn, kp, b, h)) != cudaSuccess)
         return done(e);
       last = wn;
     }
