@@ -399,8 +399,6 @@ void ensure_graphs(ehd_sim* s) {
   s->mgraphs_ok = mok;
 }
 
-// Copies one input field into the staging area; returns its largest magnitude in *amax
-// (used to choose the FP16 storage scales).
 // dst[j][i] = (To)src[j][i] for j < nf, i < n: the conversions between the caller's
 // double arrays and the float32 staging buffers, split over up to 8 host threads when
 // there are at least 2^20 values in all (below that, starting threads costs more than
@@ -431,31 +429,39 @@ void convert(To* const* dst, const From* const* src, int nf, size_t n) {
   for (auto& x : th) x.join();
 }
 
-int stage_in(ehd_sim* s, const void* src, int slot, int mem, double* amax) {
+// Copies one input field into the staging area.
+int stage_in(ehd_sim* s, const void* src, int slot, int mem) {
   const size_t N = (size_t)s->kp.N;
   float* dst = s->b.io + slot * N;
-  float* stage = s->h_stage + slot * N;
   if (mem == EHD_DEVICE) {
     EHD_CUDA(cudaMemcpyAsync(dst, src, N * sizeof(float), cudaMemcpyDeviceToDevice,
                              s->stream));
-    if (s->kp.half) {
-      EHD_CUDA(cudaMemcpyAsync(stage, src, N * sizeof(float), cudaMemcpyDeviceToHost, s->stream));
-      EHD_CUDA(cudaStreamSynchronize(s->stream));
-    }
   } else {
+    float* stage = s->h_stage + slot * N;
     const double* d = static_cast<const double*>(src);
     convert(&stage, &d, 1, N);
     EHD_CUDA(cudaMemcpyAsync(dst, stage, N * sizeof(float), cudaMemcpyHostToDevice,
                              s->stream));
   }
-  double m = 0.0;
-  if (s->kp.half)
-    for (size_t i = 0; i < N; ++i) {
-      const double a = std::fabs((double)stage[i]);
-      m = a > m ? a : m;
-    }
-  *amax = m;
   return EHD_OK;
+}
+
+// Whether a kernel on the current device may write float32 arrays at these addresses: device
+// memory of this device, 4-byte aligned.  (What else a caller calls a device array goes through
+// a copy, which reports what it cannot reach.)
+bool writable_here(void* const* out, int n) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  for (int j = 0; j < n; ++j) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, out[j]) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (a.type != cudaMemoryTypeDevice || a.device != dev || (reinterpret_cast<uintptr_t>(out[j]) & 3u))
+      return false;
+  }
+  return true;
 }
 
 // Power of two 2^floor(log2(1/ref)): the FP16 scale that maps a magnitude ref to [0.5, 1).
@@ -732,8 +738,10 @@ int ehd_solve_potential(ehd_sim* s, double tol, int max_iter, int* iters, double
                                    s->stream, s->resident_ok));
   int st = run_potential_loop(s, fixed, mx);
   if (st == EHD_ERR_CUDA) return st;
-  EHD_CUDA(cudaMemcpyAsync(s->h_ctl, s->b.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s->stream));
-  EHD_CUDA(cudaStreamSynchronize(s->stream));
+  if (!s->resident_ok && fixed > 0) {  // the other loops end with the control read back
+    EHD_CUDA(cudaMemcpyAsync(s->h_ctl, s->b.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s->stream));
+    EHD_CUDA(cudaStreamSynchronize(s->stream));
+  }
   if (iters) *iters = s->h_ctl->iter;
   if (rel_change) *rel_change = s->h_ctl->rel;
   if (s->h_ctl->nonfinite) return EHD_ERR_NONFINITE;
@@ -746,17 +754,25 @@ int ehd_set_fields(ehd_sim* s, const void* phi, const void* q, const void* ux, c
     return EHD_ERR_INVALID_ARG;
   NvtxRange range("ehd_set_fields");
   int st;
-  double m_phi, m_q, m_ux, m_uy, m_p;
-  if ((st = stage_in(s, phi, 0, mem, &m_phi)) != EHD_OK) return st;
-  if ((st = stage_in(s, q, 1, mem, &m_q)) != EHD_OK) return st;
-  if ((st = stage_in(s, ux, 2, mem, &m_ux)) != EHD_OK) return st;
-  if ((st = stage_in(s, uy, 3, mem, &m_uy)) != EHD_OK) return st;
-  if (p && (st = stage_in(s, p, 4, mem, &m_p)) != EHD_OK) return st;
+  const void* in[5] = {phi, q, ux, uy, p};
+  for (int j = 0; j < 5; ++j)
+    if (in[j] && (st = stage_in(s, in[j], j, mem)) != EHD_OK) return st;
   if (s->kp.half) {
-    choose_scales(s, m_q, m_ux > m_uy ? m_ux : m_uy);
-    // the step graphs hold the coefficients: rebuild them with the new scales
-    destroy_graphs(s);
-    s->graphs_tried = false;
+    unsigned* amax = reinterpret_cast<unsigned*>(s->b.partials);
+    EHD_CUDA(launch_absmax(s->kp, s->b, amax, s->stream));
+    EHD_CUDA(cudaMemcpyAsync(s->h_stats, amax, 3 * sizeof(unsigned), cudaMemcpyDeviceToHost,
+                             s->stream));
+    EHD_CUDA(cudaStreamSynchronize(s->stream));
+    float m[3];  // of q, ux, uy
+    std::memcpy(m, s->h_stats, sizeof(m));
+    float old[3];
+    std::memcpy(old, s->kp.psc, sizeof(old));
+    choose_scales(s, m[0], m[1] > m[2] ? m[1] : m[2]);
+    // the step graphs hold the coefficients: they stay where the scales, powers of two, do
+    if (std::memcmp(old, s->kp.psc, sizeof(old)) != 0) {
+      destroy_graphs(s);
+      s->graphs_tried = false;
+    }
   }
   s->n = s->P.start_step;
   s->history_valid = false;
@@ -922,8 +938,16 @@ int ehd_read_fields(ehd_sim* s, unsigned mask, void* const* out, int mem) {
       if (!out[nf]) return EHD_ERR_INVALID_ARG;
       ++nf;
     }
-  EHD_CUDA(launch_fields(s->kp, s->b, s->cur, mask, s->stream));
   const size_t N = (size_t)s->kp.N;
+  if (mem == EHD_DEVICE && writable_here(out, nf)) {
+    // straight into the caller's arrays
+    float* outs[EHD_NUM_FIELDS];
+    for (int j = 0; j < nf; ++j) outs[j] = static_cast<float*>(out[j]);
+    EHD_CUDA(launch_fields(s->kp, s->b, s->cur, mask, s->stream, outs));
+    EHD_CUDA(cudaStreamSynchronize(s->stream));
+    return EHD_OK;
+  }
+  EHD_CUDA(launch_fields(s->kp, s->b, s->cur, mask, s->stream));
   for (int j = 0; j < nf; ++j) {
     if (mem == EHD_DEVICE) {
       EHD_CUDA(cudaMemcpyAsync(out[j], s->b.io + j * N, N * sizeof(float),
@@ -1022,7 +1046,7 @@ int ehd_load_state(ehd_sim* s, const void* buf, size_t bytes) {
   const size_t N = (size_t)s->kp.N;
   const char* p = static_cast<const char*>(buf) + sizeof(hd);
   s->cur = 0;
-  if (s->kp.half) {
+  if (s->kp.half && std::memcmp(s->kp.psc, hd.psc, sizeof(hd.psc)) != 0) {
     for (int f = 0; f < 3; ++f) {
       s->kp.psc[f] = hd.psc[f];
       s->kp.ipsc[f] = 1.0f / hd.psc[f];

@@ -495,6 +495,11 @@ struct Buffers {
   float2* rpartials; // resident loop: [2][tiles] float2; D-step loop: [2][tiles][D / 2 + D % 2] float4
 };
 
+// The arrays an output pass writes, in the order of the mask's bits.
+struct FieldOut {
+  float* p[NIO];
+};
+
 __host__ __device__ inline Pops pops_copy(const KParams& k, const Buffers& b, int c) {
   Pops P;
   if (k.half) {
@@ -599,14 +604,17 @@ cudaError_t launch_poisson(const KParams& kp, const Buffers& b, cudaStream_t st)
 cudaError_t launch_coupled(const KParams& kp, const Buffers& b, int cur, cudaStream_t st);
 cudaError_t launch_stats_reset(const Buffers& b, cudaStream_t st);
 cudaError_t launch_expire_barrier(const Buffers& b, cudaStream_t st);
+// The requested fields into the caller's device arrays `outs` (in mask order), or with null
+// `outs` into the staging slots.
 cudaError_t launch_fields(const KParams& kp, const Buffers& b, int cur, unsigned mask,
-                          cudaStream_t st);
+                          cudaStream_t st, float* const* outs = nullptr);
+cudaError_t launch_absmax(const KParams& kp, const Buffers& b, unsigned* out, cudaStream_t st);
 cudaError_t launch_phi_now(const KParams& kp, const Buffers& b, int cur, cudaStream_t st);
 // The contact line on the bottom wall into b.partials[0..1] (see k_contact_line).
 cudaError_t launch_contact_line(const KParams& kp, const Buffers& b, int cur, float level,
                                 cudaStream_t st);
 cudaError_t launch_fields_from_phi(const KParams& kp, const Buffers& b, int cur, unsigned mask,
-                                   cudaStream_t st);
+                                   cudaStream_t st, float* const* outs = nullptr);
 cudaError_t add_poisson_node_nocond(cudaGraph_t g, const cudaGraphNode_t* deps, size_t nd,
                                     cudaGraphNode_t* out, const KParams& kp, const Buffers& b);
 

@@ -1026,7 +1026,7 @@ template <bool HALF>
 __global__ void k_fields(KParams k, const StepState* __restrict__ ss, Pops pops,
                          const float* __restrict__ phi_now, const float* __restrict__ phi_solve,
                          const float* __restrict__ hbuf, const float* __restrict__ hist,
-                         const Ctl* ctl, unsigned mask, float* __restrict__ io) {
+                         const Ctl* ctl, unsigned mask, FieldOut out) {
   const int N = k.N;
   const int i0 = blockIdx.x * blockDim.x + threadIdx.x;
   if (i0 >= k.nint) return;
@@ -1085,7 +1085,7 @@ __global__ void k_fields(KParams k, const StepState* __restrict__ ss, Pops pops,
 #pragma unroll
   for (int b = 0; b < NIO; ++b) {
     if (mask & (1u << b)) {
-      io[slot * (size_t)N + idx] = vals[b];
+      out.p[slot][idx] = vals[b];
       ++slot;
     }
   }
@@ -1164,18 +1164,45 @@ cudaError_t launch_stats_reset(const Buffers& b, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+// Where the requested fields go: the caller's arrays (`outs`, in mask order) or, with a null
+// `outs`, the staging slots.
+static FieldOut field_out(const KParams& kp, const Buffers& b, float* const* outs, unsigned mask) {
+  FieldOut o{};
+  int n = 0;
+  for (int f = 0; f < NIO; ++f)
+    if (mask & (1u << f)) {
+      o.p[n] = outs ? outs[n] : b.io + (size_t)n * kp.N;
+      ++n;
+    }
+  return o;
+}
+
 cudaError_t launch_fields(const KParams& kp, const Buffers& b, int cur, unsigned mask,
-                          cudaStream_t st) {
-  const Pops P = pops_copy(kp, b, cur);
-  if (kp.half) {
-    k_phi_now<true><<<blocks_for(kp.nint, 256), 256, 0, st>>>(kp, P, b.tmp);
-    k_fields<true><<<blocks_for(kp.nint, 256), 256, 0, st>>>(kp, b.ss + cur, P, b.tmp, b.phi, b.h,
-                                                          b.hist, b.ctl, mask, b.io);
-  } else {
-    k_phi_now<false><<<blocks_for(kp.nint, 256), 256, 0, st>>>(kp, P, b.tmp);
-    k_fields<false><<<blocks_for(kp.nint, 256), 256, 0, st>>>(kp, b.ss + cur, P, b.tmp, b.phi,
-                                                           b.h, b.hist, b.ctl, mask, b.io);
-  }
+                          cudaStream_t st, float* const* outs) {
+  const cudaError_t e = launch_phi_now(kp, b, cur, st);
+  if (e != cudaSuccess) return e;
+  return launch_fields_from_phi(kp, b, cur, mask, st, outs);
+}
+
+// The largest magnitudes of the staged q, ux and uy (slots 1 to 3; NaNs aside), which the
+// FP16 storage scales come from, as the bits of non-negative floats in out[0..2] (zeroed).  One
+// read of three fields, where the host used to copy every field back and walk over it (0.8 ms
+// of a set-up at 512 x 1024).
+__global__ void __launch_bounds__(256) k_absmax(const float* __restrict__ io, int N, unsigned* out) {
+  const float* v = io + (size_t)(1 + blockIdx.y) * N;
+  float m = 0.0f;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x)
+    m = fmaxf(m, fabsf(__ldg(v + i)));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) atomicMax(out + blockIdx.y, __float_as_uint(m));
+}
+
+cudaError_t launch_absmax(const KParams& kp, const Buffers& b, unsigned* out, cudaStream_t st) {
+  const cudaError_t e = cudaMemsetAsync(out, 0, 3 * sizeof(unsigned), st);
+  if (e != cudaSuccess) return e;
+  const int nb = blocks_for(kp.N, 256) < 304 ? blocks_for(kp.N, 256) : 304;
+  k_absmax<<<dim3(nb, 3), 256, 0, st>>>(b.io, kp.N, out);
   return cudaGetLastError();
 }
 
@@ -1190,14 +1217,15 @@ cudaError_t launch_phi_now(const KParams& kp, const Buffers& b, int cur, cudaStr
   return cudaGetLastError();
 }
 cudaError_t launch_fields_from_phi(const KParams& kp, const Buffers& b, int cur, unsigned mask,
-                                   cudaStream_t st) {
+                                   cudaStream_t st, float* const* outs) {
   const Pops P = pops_copy(kp, b, cur);
+  const FieldOut o = field_out(kp, b, outs, mask);
   if (kp.half)
     k_fields<true><<<blocks_for(kp.nint, 256), 256, 0, st>>>(kp, b.ss + cur, P, b.tmp, b.phi, b.h,
-                                                             b.hist, b.ctl, mask, b.io);
+                                                             b.hist, b.ctl, mask, o);
   else
     k_fields<false><<<blocks_for(kp.nint, 256), 256, 0, st>>>(kp, b.ss + cur, P, b.tmp, b.phi,
-                                                              b.h, b.hist, b.ctl, mask, b.io);
+                                                              b.h, b.hist, b.ctl, mask, o);
   return cudaGetLastError();
 }
 
