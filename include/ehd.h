@@ -52,9 +52,12 @@ typedef enum ehd_status {
 enum { EHD_HOST = 0, EHD_DEVICE = 1 };
 enum { EHD_FP32 = 0, EHD_FP16DEV = 1 };
 /* Implementation of the potential sub-iteration loop (same arithmetic, same results):
- * STREAM runs one kernel per sub-iteration over populations in device memory; RESIDENT
- * runs the whole loop in one cooperative kernel with the populations held on chip (only
- * for lattices that fit, about 600k nodes on a GB300); AUTO picks RESIDENT when it fits. */
+ * STREAM runs kernels over populations in device memory, one per sub-iteration (above 600k
+ * nodes up to five sub-iterations per kernel); RESIDENT runs the whole loop in one kernel
+ * with the populations held on chip (only for lattices that fit, about 600k nodes on a
+ * GB300; with the library's own tiles, lattices up to about 46k nodes run on one
+ * thread-block cluster); AUTO picks RESIDENT where it fits, RESIDENT2 where that fits the
+ * same tiles beyond one cluster. */
 enum {
   EHD_LOOP_AUTO = 0,
   EHD_LOOP_STREAM = 1,

@@ -83,6 +83,11 @@ Layout layout_for(const ehd_params& P, int fixed_ty = 0) {
   if (resident_geometry(kp, device_sms(), &g, &th, &sm, fixed_ty, loop_depth(P.poisson_loop))) {
     L.rtiles = (size_t)g.ntx * g.nty;
     L.export_floats = 2 * L.rtiles * 8 * (size_t)g.pmax;
+    // the library's own choice may be the two-step loop on the same tiles (wider bands)
+    if (P.poisson_loop == EHD_LOOP_AUTO && fixed_ty == 0 &&
+        resident_geometry(kp, device_sms(), &g, &th, &sm, 0, 2) &&
+        (size_t)g.ntx * g.nty == L.rtiles && 2 * L.rtiles * 8 * (size_t)g.pmax > L.export_floats)
+      L.export_floats = 2 * L.rtiles * 8 * (size_t)g.pmax;
   }
   L.exports = take(sizeof(float) * (L.export_floats ? L.export_floats : 1));
   // [2][tiles] float2 partial sums (multi-step loop: [2][tiles] one or two float4,
@@ -592,20 +597,21 @@ int sim_create(const ehd_params* params, void* workspace, size_t workspace_bytes
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess &&
         coop && L.export_floats && params->poisson_loop != EHD_LOOP_STREAM) {
-      const int use_sms = sms;
+      // the conventional scheme runs on the one- and two-step loops
+      const bool conv = params->potential_scheme == EHD_SCHEME_CONVENTIONAL;
       ResidentGeom g;
       int th;
       size_t sm;
-      const int depth = loop_depth(params->poisson_loop);
-      // the conventional scheme runs on the one- and two-step loops
-      const bool conv = params->potential_scheme == EHD_SCHEME_CONVENTIONAL;
-      const void* fk = nullptr;
-      if (resident_geometry(s->kp, use_sms, &g, &th, &sm, fixed_ty, depth) &&
-          (fk = resident_kernel(g.TY, depth, conv)) != nullptr &&
-          2 * (size_t)g.ntx * g.nty * 8 * g.pmax <= L.export_floats &&
-          (size_t)g.ntx * g.nty <= L.rtiles &&
-          cudaFuncSetAttribute(fk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) ==
-              cudaSuccess) {
+      // whether the tiled loop of that many sub-iterations per exchange fits on chip
+      auto fits = [&](int depth) {
+        const void* fk = nullptr;
+        if (!resident_geometry(s->kp, sms, &g, &th, &sm, fixed_ty, depth) ||
+            (fk = resident_kernel(g.TY, depth, conv)) == nullptr ||
+            2 * (size_t)g.ntx * g.nty * 8 * g.pmax > L.export_floats ||
+            (size_t)g.ntx * g.nty > L.rtiles ||
+            cudaFuncSetAttribute(fk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) !=
+                cudaSuccess)
+          return false;
         int per_sm = 0;
         // the multi-step loops hold tensor memory for the whole launch: CTAs that share
         // an SM must fit its 512 columns together, or a CTA would wait in tcgen05.alloc
@@ -615,21 +621,39 @@ int sim_create(const ehd_params* params, void* workspace, size_t workspace_bytes
           per_sm = 0;
         if (tcols < 0) per_sm = 0;
         if (tcols > 0 && per_sm > 512 / tcols) per_sm = 512 / tcols;
-        if (per_sm >= 1 && (long long)g.ntx * g.nty <= (long long)per_sm * sms) {
-          s->resident_ok = true;
-          s->rg = g;
-          s->rthreads = th;
-          s->rsmem = sm;
-          // the library's own choice of tiles: a lattice that fits one cluster's shared
-          // memory runs its loop there (the tiles stay laid out for the diagnostics)
-          ClusterGeom cg;
-          if (depth == 0 && fixed_ty == 0)
-            for (int most = 16; most >= 8; most -= 8)
-              if (cluster_geometry(s->kp, &cg, most) && cluster_usable(s->kp, cg)) {
-                s->rg.cluster = cg;
-                break;
-              }
-        }
+        return per_sm >= 1 && (long long)g.ntx * g.nty <= (long long)per_sm * sms;
+      };
+      auto take = [&]() {
+        s->resident_ok = true;
+        s->rg = g;
+        s->rthreads = th;
+        s->rsmem = sm;
+      };
+      const int depth = loop_depth(params->poisson_loop);
+      if (fits(depth)) {
+        take();
+        // the library's own choice of tiles: a lattice that fits one cluster's shared
+        // memory runs its loop there (the tiles stay laid out for the diagnostics)
+        ClusterGeom cg;
+        if (depth == 0 && fixed_ty == 0)
+          for (int most = 16; most >= 8; most -= 8)
+            if (cluster_geometry(s->kp, &cg, most) && cluster_usable(s->kp, cg)) {
+              s->rg.cluster = cg;
+              break;
+            }
+        // and the other lattices run two sub-iterations per exchange where that fits the same
+        // tiles, whose sums and so decisions are the one-step loop's bit for bit.  Per step at
+        // K = 2 and 5 it takes 23.9 and 32.8 us against 28.0 and 39.1 at 256 x 256, 49.8 and 63.1
+        // against 51.3 and 63.8 at 512 x 1024.  A cycle makes two sub-iterations whether the
+        // second is wanted or not: with tiles above 32 rows a fixed count of 1 (37.2 against
+        // 35.9 us at 512 x 700), with 48 and more also one of 3 (56.6 against 55.4 at
+        // 512 x 1024), stays with the one-step loop.
+        const ResidentGeom one = g;
+        const int k = params->poisson_fixed_iter;
+        if (params->poisson_loop == EHD_LOOP_AUTO && fixed_ty == 0 && s->rg.cluster.size == 0 &&
+            !(one.TY > 32 && k == 1) && !(one.TY >= 48 && k == 3) && fits(2) && g.TY == one.TY &&
+            g.nty == one.nty)
+          take();
       }
     }
     cudaGetLastError();

@@ -24,7 +24,7 @@ SHAPES = [(16, 32),    # 1, 32, 512
           (180, 149),  # 15, 10, 1920
           (187, 194),  # 15, 13, 2432
           (180, 256),  # 16, 16, 2880
-          (181, 256)]  # tiled
+          (181, 256)]  # beyond: the two-step tiled loop (a count of 1: the one-step loop)
 
 
 @pytest.fixture(scope="module")
@@ -76,7 +76,7 @@ def test_fixed_count_equals_streaming(gpu, nx, ny, walls, scheme):
         p, f = setup(nx, ny, walls, scheme, poisson_fixed_iter=k)
         a, ia, kind = states(gpu, p, f, 2)
         b, ib, _ = states(gpu, dict(p, poisson_loop=1), f, 2)
-        assert kind == 2 and ia == ib == 2 * k
+        assert kind == (3 if nx == 181 and k > 1 else 2) and ia == ib == 2 * k
         for name in a:
             assert np.array_equal(a[name], b[name]), (name, k)
 
