@@ -759,7 +759,7 @@ int ehd_solve_potential(ehd_sim* s, double tol, int max_iter, int* iters, double
   const int mx = max_iter > 0 ? max_iter : P.poisson_max_iter;
   const int fixed = (tol > 0 || max_iter > 0) ? 0 : P.poisson_fixed_iter;
   EHD_LAUNCH(s, 0, launch_moments(s->kp, s->b, s->cur, t, P.poisson_min_iter, mx, fixed,
-                                   s->stream, s->resident_ok));
+                                   s->stream, s->resident_ok || multi_defers(s->kp)));
   int st = run_potential_loop(s, fixed, mx);
   if (st == EHD_ERR_CUDA) return st;
   if (!s->resident_ok && fixed > 0) {  // the other loops end with the control read back
@@ -894,7 +894,8 @@ int ehd_step(ehd_sim* s, int nsteps, ehd_stats* out) {
         NvtxRange r("moments");
         EHD_LAUNCH(s, 0, launch_moments(s->kp, s->b, s->cur, P.poisson_tol,
                                          P.poisson_min_iter, P.poisson_max_iter,
-                                         P.poisson_fixed_iter, s->stream, s->resident_ok));
+                                         P.poisson_fixed_iter, s->stream,
+                                         s->resident_ok || multi_defers(s->kp)));
       }
       int st;
       {

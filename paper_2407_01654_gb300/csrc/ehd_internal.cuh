@@ -543,6 +543,7 @@ struct StepSlot {
 __host__ __device__ inline bool moments4_ok(const KParams& kp) {
   return !kp.slab && kp.N % 4 == 0 && kp.N == kp.nint;
 }
+__host__ __device__ inline int moments4_blocks(const KParams& kp) { return (kp.N / 4 + 255) / 256; }
 
 // Batched moments / coupled passes: one launch over work[] = (slot, block of that slot).
 cudaError_t add_moments_batch_node(cudaGraph_t g, const cudaGraphNode_t* deps, size_t nd,
@@ -574,6 +575,7 @@ cudaError_t add_poisson_resident_node(cudaGraph_t graph, const cudaGraphNode_t* 
 // Streaming with several sub-iterations per launch (poisson_multi.cu).
 constexpr long long MULTI_MIN_NODES = 600000;
 bool multi_ok(const KParams& kp);
+bool multi_defers(const KParams& kp);
 cudaError_t multi_prepare(const KParams& kp);
 int multi_launches(int fixed);  // launches of a fixed count
 cudaError_t launch_poisson_multi(const KParams& kp, const Buffers& b, cudaStream_t st);
@@ -595,8 +597,8 @@ cudaError_t launch_step_set(const KParams& kp, const Buffers& b, int slot, long 
                             int first, cudaStream_t st);
 cudaError_t launch_init(const KParams& kp, const Buffers& b, int cur, bool have_p,
                         cudaStream_t st);
-// sums_in_coupled: the potential loop that follows runs on chip, so (without a neutralised
-// source) the moments pass may leave its FP64 sums as per-CTA partials for the coupled pass.
+// sums_in_coupled: the potential loop that follows needs no sums and leaves the partials alone
+// (on chip, or multi_defers), so (without a neutralised source) the moments pass may leave its FP64 sums as per-CTA partials for the coupled pass.
 cudaError_t launch_moments(const KParams& kp, const Buffers& b, int cur, double tol,
                            int min_iter, int max_iter, int fixed_iter, cudaStream_t st,
                            bool sums_in_coupled = false);

@@ -500,8 +500,6 @@ static inline const void* moments4_kernel(const KParams& kp, bool tail) {
     return tail ? (const void*)k_moments4<true, true> : (const void*)k_moments4<false, true>;
   return tail ? (const void*)k_moments4<true, false> : (const void*)k_moments4<false, false>;
 }
-// Whether a lattice takes k_moments4 (moments4_ok, in the header), and its grid.
-static inline int moments4_blocks(const KParams& kp) { return (kp.N / 4 + 255) / 256; }
 
 // ------------------------------------------------------------------------------------
 // The fused coupled pass (a1, a2, a4-a9): stencils on phi, field from the converged
@@ -1350,7 +1348,7 @@ cudaError_t build_step_graph(const KParams& kp, const Buffers& b, int cur, doubl
     cudaGraphNode_t mn, wn, pn, cn;
     if ((e = record(0)) != cudaSuccess ||
         (e = add_moments_node(g, have ? &last : nullptr, have ? 1 : 0, &mn, kp, b, c, tol,
-                              min_iter, max_iter, fixed_iter, rg != nullptr)) != cudaSuccess)
+                              min_iter, max_iter, fixed_iter, rg || multi_defers(kp))) != cudaSuccess)
       return done(e);
     last = mn;
     have = true;
