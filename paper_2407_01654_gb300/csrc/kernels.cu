@@ -911,9 +911,7 @@ __global__ void __launch_bounds__(256) k_moments_batch(const StepSlot* __restric
   if (S.quad && S.k.neutralize)
     S.k.half ? quad(true_type{}, true_type{}) : quad(true_type{}, false_type{});
   else if (S.quad)
-    moments4_body<true, false>(S.k, S.b.ss + cur, P, S.b.hist, S.b.phi, S.b.aq, S.b.partials,
-                               S.b.ctl, S.tol, S.min_iter, S.max_iter, S.fixed_iter, w.y,
-                               S.mblocks);
+    S.k.half ? quad(false_type{}, true_type{}) : quad(false_type{}, false_type{});
   else if (S.k.half)
     moments_body<true>(S.k, S.b.ss + cur, P, S.b.hist, S.b.phi, S.b.aq, S.b.partials, S.b.ctl,
                        S.tol, S.min_iter, S.max_iter, S.fixed_iter, w.y, S.mblocks);
