@@ -285,7 +285,8 @@ int run_potential_loop(ehd_sim* s, int fixed, int max_iter) {
   }
   const bool multi = multi_ok(s->kp);
   auto launch = [&]() {
-    return multi ? launch_poisson_multi(s->kp, s->b, s->stream) : launch_poisson(s->kp, s->b, s->stream);
+    return multi ? launch_poisson_multi(s->kp, s->b, fixed, s->stream)
+                 : launch_poisson(s->kp, s->b, s->stream);
   };
   if (fixed > 0) {
     const int n = multi ? multi_launches(fixed) : fixed;

@@ -578,10 +578,11 @@ bool multi_ok(const KParams& kp);
 bool multi_defers(const KParams& kp);
 cudaError_t multi_prepare(const KParams& kp);
 int multi_launches(int fixed);  // launches of a fixed count
-cudaError_t launch_poisson_multi(const KParams& kp, const Buffers& b, cudaStream_t st);
+// fixed: the solve's fixed count, or 0 under the rule.
+cudaError_t launch_poisson_multi(const KParams& kp, const Buffers& b, int fixed, cudaStream_t st);
 cudaError_t add_poisson_multi_node(cudaGraph_t g, const cudaGraphNode_t* deps, size_t nd,
                                    cudaGraphNode_t* out, const KParams& kp, const Buffers& b,
-                                   const cudaGraphConditionalHandle* handle);
+                                   int fixed, const cudaGraphConditionalHandle* handle);
 
 // The same loop on one thread-block cluster (poisson_cluster.cu): the geometry of a lattice,
 // false if it does not fit; whether this device can launch it; the launch and its graph node.

@@ -1360,7 +1360,7 @@ cudaError_t build_step_graph(const KParams& kp, const Buffers& b, int cur, doubl
       // a fixed count's few launches in a row, without a condition between them (after a
       // non-finite field the first one ends the loop and the others return at once)
       for (int l = 0; l < multi_launches(fixed_iter); ++l) {
-        if ((e = add_poisson_multi_node(g, &last, 1, &pn, kp, b, nullptr)) != cudaSuccess)
+        if ((e = add_poisson_multi_node(g, &last, 1, &pn, kp, b, fixed_iter, nullptr)) != cudaSuccess)
           return done(e);
         last = pn;
       }
@@ -1377,7 +1377,8 @@ cudaError_t build_step_graph(const KParams& kp, const Buffers& b, int cur, doubl
       cp.conditional.size = 1;
       if ((e = cudaGraphAddNode(&wn, g, &last, nullptr, 1, &cp)) != cudaSuccess ||
           (e = multi_ok(kp)
-                   ? add_poisson_multi_node(cp.conditional.phGraph_out[0], nullptr, 0, &pn, kp, b, &h)
+                   ? add_poisson_multi_node(cp.conditional.phGraph_out[0], nullptr, 0, &pn, kp, b,
+                                            fixed_iter, &h)
                    : add_poisson_node(cp.conditional.phGraph_out[0], &pn, kp, b, h)) != cudaSuccess)
         return done(e);
       last = wn;

@@ -19,6 +19,12 @@
 // where FP64 sums in another order do.  The last CTA applies the rule to the n sub-iterations in
 // order.  When it stops the loop before the n-th, the state in the other copy of h, from which
 // this launch began, is advanced again by that many: one more launch per solve at most.
+//
+// A fixed count needs no decision, so the order of its sums (a statistic) is free and with it
+// the tile height: two CTAs fit an SM, and tiles as tall as the lattice's whole waves of
+// 2 x 152 need (multi_rows) leave no nearly empty last wave: five sub-iterations at 977 x 811
+// take 58.9 us with 592 tiles of 22 rows against 66.1 with 416 of 32, at 1024 x 2048 118.6 with
+// 1184 of 28 rows against 120.9 with 1024 of 32.
 #include "ehd_internal.cuh"
 
 namespace ehd {
@@ -59,7 +65,7 @@ __host__ __device__ inline int multi_steps(int d, int fixed, int max_iter, int i
 
 template <int D, bool CONV>
 __global__ void __launch_bounds__(MT, 2)
-    k_poisson_multi(KParams k, float* __restrict__ hbuf, const float2* __restrict__ aq,
+    k_poisson_multi(KParams k, int th, float* __restrict__ hbuf, const float2* __restrict__ aq,
                     double2* __restrict__ partials, Ctl* ctl, cudaGraphConditionalHandle cond,
                     int use_cond) {
   using M = Multi<D>;
@@ -84,7 +90,7 @@ __global__ void __launch_bounds__(MT, 2)
   const size_t N = (size_t)k.N;
   const float* __restrict__ src = hbuf + (size_t)parity * NH * N;
   float* __restrict__ dst = hbuf + (size_t)(parity ^ 1) * NH * N;
-  const int x0 = blockIdx.x * MTX, y0 = blockIdx.y * MTY;
+  const int x0 = blockIdx.x * MTX, y0 = blockIdx.y * th;  // a 64 x th tile, th <= MTY
   const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float om = k.omega_h;
 
@@ -114,20 +120,34 @@ __global__ void __launch_bounds__(MT, 2)
     return f | (k.walls && gy == 0 ? W_BOT : 0u) | (k.walls && gy == ny - 1 ? W_TOP : 0u);
   };
 
-  // my tile nodes: column lx, rows ly + 2 j of a 16-row block
+  // my tile nodes, in column lx: of a full tile the rows ly + 2 j of a 16-row block (the
+  // one-step kernel's sums); of a lower one pairs of rows, dealt in turn to the four rows of
+  // threads, so that all have alike much to do
+  const bool full = th == MTY;
   const int lx = tid & 63, ly = (tid >> 7) * 16 + ((tid >> 6) & 1);
+  auto row_of = [&](int j) {
+    return full ? ly + 2 * j : 2 * ((tid >> 6) + 4 * (j >> 1)) + (j & 1);
+  };
   unsigned tf[MNODE];
   float2 ta[MNODE / 2], tq[MNODE / 2];
 #pragma unroll
-  for (int j = 0; j < MNODE; ++j)
-    tf[j] = (j & 1) ? fetch(lx, ly + 2 * j, ta[j >> 1].y, tq[j >> 1].y)
-                    : fetch(lx, ly + 2 * j, ta[j >> 1].x, tq[j >> 1].x);
+  for (int j = 0; j < MNODE; ++j) {
+    float a = 0.0f, q = 0.0f;
+    tf[j] = row_of(j) < th ? fetch(lx, row_of(j), a, q) : W_NONE;
+    if (j & 1) {
+      ta[j >> 1].y = a;
+      tq[j >> 1].y = q;
+    } else {
+      ta[j >> 1].x = a;
+      tq[j >> 1].x = q;
+    }
+  }
   // my nodes of the ring, n wide: n rows below, n above (each 64 + 2 n long), then n columns on
   // either side; the layer (1 next to the tile) above the wall bits
   unsigned rf[2 * M::PAIRS];
   float2 ra[M::PAIRS], rq[M::PAIRS];
   {
-    const int wide = MTX + 2 * n, rows = 2 * n * wide, ring = rows + 2 * n * MTY;
+    const int wide = MTX + 2 * n, rows = 2 * n * wide, ring = rows + 2 * n * th;
 #pragma unroll
     for (int m = 0; m < 2 * M::PAIRS; ++m) {
       const int r = tid + m * MT;
@@ -138,14 +158,14 @@ __global__ void __launch_bounds__(MT, 2)
         if (r < rows) {
           const int row = r / wide;
           x = r - row * wide - n;
-          y = row < n ? row - n : MTY + row - n;
+          y = row < n ? row - n : th + row - n;
         } else {
-          const int c = (r - rows) / MTY;
-          y = (r - rows) - c * MTY;
+          const int c = (r - rows) / th;
+          y = (r - rows) - c * th;
           x = c < n ? c - n : MTX + c - n;
         }
         const int dx = x < 0 ? -x : (x >= MTX ? x - MTX + 1 : 0);
-        const int dy = y < 0 ? -y : (y >= MTY ? y - MTY + 1 : 0);
+        const int dy = y < 0 ? -y : (y >= th ? y - th + 1 : 0);
         w = fetch(x, y, a, q) | ((unsigned)(dx > dy ? dx : dy) << 20);
       }
       rf[m] = w;
@@ -210,8 +230,8 @@ __global__ void __launch_bounds__(MT, 2)
   auto add_sums = [&](int j, float2 v, float& num, float& den) {
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-      const int gy = y0 + ly + 2 * (2 * j + c);
-      if (x0 + lx < nx && gy < ny)
+      const int y = row_of(2 * j + c);
+      if (x0 + lx < nx && y < th && y0 + y < ny)
         h_change(c ? v.y : v.x, c ? vold[j].y : vold[j].x, num, den);
     }
   };
@@ -226,13 +246,14 @@ __global__ void __launch_bounds__(MT, 2)
   // A CTA away from the walls (mask: only the frame index of a tile node counts) runs code
   // without a wall in it: the walled form is several times as long, more than the instruction
   // cache close to the issue slots holds.
-  const bool near_wall = k.walls && (y0 - n <= 0 || y0 + MTY + n >= ny);
+  const bool near_wall = k.walls && (y0 - n <= 0 || y0 + th + n >= ny);
   auto sub_iteration = [&](int u, bool sw, unsigned mask) {
     float num = 0.0f, den = 0.0f;
 #pragma unroll
     for (int j = 0; j < MNODE / 2; ++j) {
       float2 h[8];
       const unsigned t0 = tf[2 * j] & mask, t1 = tf[2 * j + 1] & mask;
+      if ((t0 & W_NONE) && (t1 & W_NONE)) continue;
       read_pair(t0, t1, sw, h);
       const float2 hsum = h_sum8x2(h);
       // (scalar products: a packed one may be contracted with the subtraction of its old value)
@@ -267,7 +288,7 @@ __global__ void __launch_bounds__(MT, 2)
   if (near_wall)
     sub_iterations(0xfffffu);
   else
-    sub_iterations(0xffffu);
+    sub_iterations(0xffffu | W_NONE);
 
   // the new state of the tile, to the other copy of h
   {
@@ -279,8 +300,8 @@ __global__ void __launch_bounds__(MT, 2)
         read_pair(tf[2 * j] & mask, tf[2 * j + 1] & mask, sw, h);
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
-          const int gy = y0 + ly + 2 * (2 * j + c);
-          if (x0 + lx >= nx || gy >= ny) continue;
+          const int y = row_of(2 * j + c), gy = y0 + y;
+          if (x0 + lx >= nx || y >= th || gy >= ny) continue;
           const size_t g = EHD_IDX(k, (size_t)gy * nx + x0 + lx, N);
 #pragma unroll
           for (int i = 0; i < 8; ++i) dst[i * N + g] = c ? h[i].y : h[i].x;
@@ -402,9 +423,33 @@ namespace {
 #define EHD_MULTI_D 5
 #endif
 constexpr int MULTI_D = EHD_MULTI_D;
+constexpr long long MULTI_WAVE = 304;  // CTAs on the chip at once: two on each of 152 SMs
 
+dim3 multi_grid(const KParams& kp, int th) {
+  return dim3((kp.nx + MTX - 1) / MTX, (kp.ny + th - 1) / th);
+}
+// The tile height for a fixed count: the one whose waves of resident CTAs take least, a CTA's
+// time going with its tile and half the ring.  Under the rule full tiles, whose sums are the
+// one-step kernel's.
+int multi_rows(const KParams& kp, int fixed) {
+  if (fixed <= 0) return MTY;
+  const int depth = fixed < EHD_MULTI_D ? fixed : EHD_MULTI_D;
+  int best = MTY;
+  long long best_cost = -1;
+  for (int th = MTY; th >= MTY / 2; th -= 2) {  // whole pairs of rows; full tiles where equal
+    const dim3 g = multi_grid(kp, th);
+    const long long waves = ((long long)g.x * g.y + MULTI_WAVE - 1) / MULTI_WAVE;
+    const long long cost = waves * (th + depth);
+    if (best_cost < 0 || cost < best_cost) {
+      best = th;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
 int multi_blocks(const KParams& kp) {
-  return ((kp.nx + MTX - 1) / MTX) * ((kp.ny + MTY - 1) / MTY);
+  const dim3 g = multi_grid(kp, MTY);
+  return (int)(g.x * g.y);
 }
 const void* multi_kernel(const KParams& kp) {
   return kp.scheme == 1 ? (const void*)k_poisson_multi<MULTI_D, true>
@@ -414,52 +459,12 @@ const void* multi_kernel(const KParams& kp) {
 }  // namespace
 
 // Lattices that stream several sub-iterations per launch: those beyond the chip's storage, as
-// long as the partial sums of every sub-iteration of a launch have room.
+// long as the partial sums of every sub-iteration of a launch have room (a fixed count's lower
+// tiles, at most three times as many, keep only one sub-iteration's).
 bool multi_ok(const KParams& kp) {
   return !kp.slab && (long long)kp.nx * kp.ny > MULTI_MIN_NODES &&
          (long long)multi_blocks(kp) * MULTI_D <= MAX_PARTIALS;
 }
-cudaError_t multi_prepare(const KParams& kp) {
-  return cudaFuncSetAttribute(multi_kernel(kp), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)Multi<MULTI_D>::SMEM);
-}
-int multi_launches(int fixed) { return (fixed + MULTI_D - 1) / MULTI_D; }
-
-cudaError_t launch_poisson_multi(const KParams& kp, const Buffers& b, cudaStream_t st) {
-  KParams k = kp;
-  float* h = b.h;
-  const float2* aq = b.aq;
-  double2* partials = b.partials + (MAX_PARTIALS - multi_blocks(kp) * MULTI_D);
-  Ctl* ctl = b.ctl;
-  cudaGraphConditionalHandle cond = 0;
-  int use = 0;
-  void* args[] = {&k, &h, &aq, &partials, &ctl, &cond, &use};
-  return cudaLaunchKernel(multi_kernel(kp), dim3((kp.nx + MTX - 1) / MTX, (kp.ny + MTY - 1) / MTY),
-                          dim3(MT), args, Multi<MULTI_D>::SMEM, st);
-}
-
-// With a null `cond` the node leaves no condition (a fixed count's launches in a row).
-cudaError_t add_poisson_multi_node(cudaGraph_t g, const cudaGraphNode_t* deps, size_t nd,
-                                   cudaGraphNode_t* out, const KParams& kp, const Buffers& b,
-                                   const cudaGraphConditionalHandle* handle) {
-  KParams k = kp;
-  float* h = b.h;
-  const float2* aq = b.aq;
-  double2* partials = b.partials + (MAX_PARTIALS - multi_blocks(kp) * MULTI_D);
-  Ctl* ctl = b.ctl;
-  cudaGraphConditionalHandle cond = handle ? *handle : 0;
-  int use = handle ? 1 : 0;
-  void* args[] = {&k, &h, &aq, &partials, &ctl, &cond, &use};
-  cudaKernelNodeParams p = {};
-  p.func = const_cast<void*>(multi_kernel(kp));
-  p.gridDim = dim3((kp.nx + MTX - 1) / MTX, (kp.ny + MTY - 1) / MTY);
-  p.blockDim = dim3(MT);
-  p.sharedMemBytes = (unsigned)Multi<MULTI_D>::SMEM;
-  p.kernelParams = args;
-  return cudaGraphAddKernelNode(out, g, deps, nd, &p);
-}
-
-}  // namespace ehd
 // Whether the moments pass before the loop may leave its per-CTA partials to the coupled pass:
 // they keep the front of the array, the loop's sums its end (the moments pass at 1024 x 2048 went
 // from 49.3 to 37.8 us without the tickets and the last CTA's reduction).
@@ -467,3 +472,46 @@ bool multi_defers(const KParams& kp) {
   return multi_ok(kp) && moments4_ok(kp) &&
          moments4_blocks(kp) + (long long)multi_blocks(kp) * MULTI_D <= MAX_PARTIALS;
 }
+cudaError_t multi_prepare(const KParams& kp) {
+  return cudaFuncSetAttribute(multi_kernel(kp), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)Multi<MULTI_D>::SMEM);
+}
+int multi_launches(int fixed) { return (fixed + MULTI_D - 1) / MULTI_D; }
+
+cudaError_t launch_poisson_multi(const KParams& kp, const Buffers& b, int fixed, cudaStream_t st) {
+  KParams k = kp;
+  int th = multi_rows(kp, fixed);
+  float* h = b.h;
+  const float2* aq = b.aq;
+  double2* partials = b.partials + (MAX_PARTIALS - multi_blocks(kp) * MULTI_D);
+  Ctl* ctl = b.ctl;
+  cudaGraphConditionalHandle cond = 0;
+  int use = 0;
+  void* args[] = {&k, &th, &h, &aq, &partials, &ctl, &cond, &use};
+  return cudaLaunchKernel(multi_kernel(kp), multi_grid(kp, th), dim3(MT), args,
+                          Multi<MULTI_D>::SMEM, st);
+}
+
+// With a null `cond` the node leaves no condition (a fixed count's launches in a row).
+cudaError_t add_poisson_multi_node(cudaGraph_t g, const cudaGraphNode_t* deps, size_t nd,
+                                   cudaGraphNode_t* out, const KParams& kp, const Buffers& b,
+                                   int fixed, const cudaGraphConditionalHandle* handle) {
+  KParams k = kp;
+  int th = multi_rows(kp, fixed);
+  float* h = b.h;
+  const float2* aq = b.aq;
+  double2* partials = b.partials + (MAX_PARTIALS - multi_blocks(kp) * MULTI_D);
+  Ctl* ctl = b.ctl;
+  cudaGraphConditionalHandle cond = handle ? *handle : 0;
+  int use = handle ? 1 : 0;
+  void* args[] = {&k, &th, &h, &aq, &partials, &ctl, &cond, &use};
+  cudaKernelNodeParams p = {};
+  p.func = const_cast<void*>(multi_kernel(kp));
+  p.gridDim = multi_grid(kp, th);
+  p.blockDim = dim3(MT);
+  p.sharedMemBytes = (unsigned)Multi<MULTI_D>::SMEM;
+  p.kernelParams = args;
+  return cudaGraphAddKernelNode(out, g, deps, nd, &p);
+}
+
+}  // namespace ehd
