@@ -175,8 +175,9 @@ struct BatchLaunch {
   int2* work;
   StepSlot* step;
   int2* mwork;
-  int2* cwork;       // the FP32 slots' coupled blocks, then the FP16 slots'
-  int nm, nc, nc16;  // nc16 of the nc items are of FP16 slots
+  int2* cwork;
+  int nm, nc, nc16;  // nc16 of the nc coupled items are of FP16 slots
+  int nslots;
 };
 
 // Appends one batch step from copy `cur` after `dep` (null: no dependency); its last node
@@ -201,17 +202,8 @@ cudaError_t add_batch_step(cudaGraph_t g, const BatchLaunch& L, int cur,
   if ((e = cudaGraphKernelNodeSetAttribute(rn, cudaLaunchAttributeCooperative, &v)) !=
       cudaSuccess)
     return e;
-  // the coupled pass in one launch per storage precision present (the two touch
-  // disjoint slots)
-  const int n32 = L.nc - L.nc16;
-  if (n32 > 0 && L.nc16 > 0) {
-    cudaGraphNode_t c32;
-    if ((e = add_coupled_batch_node(g, &rn, 1, &c32, L.step, L.cwork, n32, cur, false)) !=
-        cudaSuccess)
-      return e;
-    return add_coupled_batch_node(g, &c32, 1, last, L.step, L.cwork + n32, L.nc16, cur, true);
-  }
-  return add_coupled_batch_node(g, &rn, 1, last, L.step, L.cwork, L.nc, cur, L.nc16 > 0);
+  return add_coupled_batch_node(g, &rn, 1, last, L.step, L.cwork, L.nc, L.nslots, cur,
+                                L.nc16 > 0);
 }
 
 // A graph of `nsteps` batch steps starting from copy `cur`, instantiated.
@@ -299,6 +291,7 @@ int rebuild(ehd_batch* b) {
   L.nm = (int)mwork.size();
   L.nc = (int)cwork.size();
   L.nc16 = nc16;
+  L.nslots = (int)live.size();
   for (int c = 0; c < 2; ++c) {
     int st = build_batch_graph(L, c, 1, &b->exec[c]);
     if (st == EHD_OK) st = build_batch_graph(L, c, b->steps_per_graph, &b->execm[c]);

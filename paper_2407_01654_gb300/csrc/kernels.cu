@@ -543,24 +543,30 @@ struct GlobalSrc {
 };
 
 // The statistics and next-step values one thread of the pass records (the potential loop
-// of this step has finished).
+// of this step has finished).  Everything is read before anything is written: one round trip
+// to L2 instead of one for each of the eight control words in turn.
 __device__ __forceinline__ void coupled_record(const KParams& k, StepState* ss, int cur,
                                                const StepState& sa, const Ctl* ctl,
                                                DevStats* stats) {
+  const int it = ld_cg(&ctl->iter), converged = ld_cg(&ctl->converged);
+  const int nonfinite = ld_cg(&ctl->nonfinite), bar_error = ld_cg(&ctl->bar_error);
+  const int plaunch = ld_cg(&ctl->plaunch);
+  const double rel = ld_cg(&ctl->rel), sum_phi = ld_cg(&ctl->sum_phi), sum_q = ld_cg(&ctl->sum_q);
+  DevStats d = *stats;
+  d.iters_total += it;
+  d.iters_min = min(d.iters_min, it);
+  d.iters_max = max(d.iters_max, it);
+  d.not_converged += converged ? 0 : 1;
+  d.nonfinite |= nonfinite;
+  d.last_rel = rel;
+  d.sum_phi = sum_phi;
+  d.sum_q = sum_q;
+  d.barrier_error |= bar_error;
+  d.plaunches += plaunch;
+  d.steps += 1;
+  *stats = d;
   // values of the next step, in the other slot (this step's slot is being read)
   ss[cur ^ 1] = make_step(k, sa.n + 1, 0);
-  const int it = ld_cg(&ctl->iter);
-  stats->iters_total += it;
-  stats->iters_min = min(stats->iters_min, it);
-  stats->iters_max = max(stats->iters_max, it);
-  stats->not_converged += ld_cg(&ctl->converged) ? 0 : 1;
-  stats->nonfinite |= ld_cg(&ctl->nonfinite);
-  stats->last_rel = ld_cg(&ctl->rel);
-  stats->sum_phi = ld_cg(&ctl->sum_phi);
-  stats->sum_q = ld_cg(&ctl->sum_q);
-  stats->barrier_error |= ld_cg(&ctl->bar_error);
-  stats->plaunches += ld_cg(&ctl->plaunch);
-  stats->steps += 1;
 }
 
 // The coupled pass at interior node (x, y), stored index idx: everything after the loads.
@@ -805,36 +811,44 @@ __device__ __forceinline__ void coupled_reduce_moments(const KParams& k,
   __syncthreads();
 }
 
+// This step's values: read by every thread and written by no CTA of the pass (it writes the
+// other state slot), so through the read-only path, one request per SM.
+__device__ __forceinline__ StepState coupled_state(const StepState* ss, int cur) {
+  const StepState* p = ss + cur;
+  StepState sa;
+  sa.n = __ldg(&p->n);
+  sa.first = __ldg(&p->first);
+  sa.pad = 0;
+  sa.cos_b = __ldg(&p->cos_b);
+  sa.cos_t = __ldg(&p->cos_t);
+  sa.vw_b = __ldg(&p->vw_b);
+  sa.vw_t = __ldg(&p->vw_t);
+  return sa;
+}
+
+// The pass's first CTA, which owns no nodes: the FP64 sums and the record.  They are a chain of
+// round trips to L2 about as long as a node's own work; ahead of the nodes of one CTA, as they
+// used to be, they were a third of the pass on a small lattice (7.7 -> 3.6 us at 4 x 64, 7.9 -> 4.7 at
+// 200 x 100, with FP16 storage 7.3 -> 4.9 at 256 x 256).
+__device__ __forceinline__ void coupled_keep(const KParams& k, StepState* ss, int cur, Ctl* ctl,
+                                             const double2* __restrict__ partials,
+                                             DevStats* stats) {
+  const StepState sa = coupled_state(ss, cur);
+  const int np = ld_cg(&ctl->mpart_n);
+  if (np > 0) coupled_reduce_moments(k, partials, np, ctl);
+  if (threadIdx.x == 0) coupled_record(k, ss, cur, sa, ctl, stats);
+}
+
 // Block `bid` of blocks of 128 threads over one simulation, one node per thread, loads
 // straight from device memory.
 template <bool HALF>
-__device__ __forceinline__ void coupled_body(const KParams& k, StepState* ss, int cur,
+__device__ __forceinline__ void coupled_body(const KParams& k, const StepState* ss, int cur,
                                              const Pops& pin, const Pops& pout,
                                              const float* __restrict__ phi_f,
                                              const float* __restrict__ hbuf,
-                                             float* __restrict__ hist, Ctl* ctl,
-                                             const double2* __restrict__ partials,
-                                             DevStats* stats, int bid) {
-  // the control words and this step's state are read by every thread and written by no
-  // CTA of the pass (it writes the other state slot): the read-only path, one request
-  // per SM
-  const int parity = __ldg(&ctl->parity);
-  StepState sa;
-  {
-    const StepState* p = ss + cur;
-    sa.n = __ldg(&p->n);
-    sa.first = __ldg(&p->first);
-    sa.pad = 0;
-    sa.cos_b = __ldg(&p->cos_b);
-    sa.cos_t = __ldg(&p->cos_t);
-    sa.vw_b = __ldg(&p->vw_b);
-    sa.vw_t = __ldg(&p->vw_t);
-  }
-  if (bid == 0) {
-    const int np = ld_cg(&ctl->mpart_n);
-    if (np > 0) coupled_reduce_moments(k, partials, np, ctl);
-    if (threadIdx.x == 0) coupled_record(k, ss, cur, sa, ctl, stats);
-  }
+                                             float* __restrict__ hist, const Ctl* ctl, int bid) {
+  const int parity = __ldg(&ctl->parity);  // as the state: read by all, written by none
+  const StepState sa = coupled_state(ss, cur);
   const int i0 = bid * blockDim.x + threadIdx.x;  // interior node
   if (i0 >= k.nint) return;
   const int y = i0 / k.nx, x = i0 - y * k.nx;
@@ -857,7 +871,10 @@ __global__ void __launch_bounds__(128) k_coupled(KParams k, StepState* ss, int c
                                                  float* __restrict__ hist, Ctl* ctl,
                                                  const double2* __restrict__ partials,
                                                  DevStats* stats) {
-  coupled_body<HALF>(k, ss, cur, pin, pout, phi_f, hbuf, hist, ctl, partials, stats, blockIdx.x);
+  if (blockIdx.x == 0)
+    coupled_keep(k, ss, cur, ctl, partials, stats);
+  else
+    coupled_body<HALF>(k, ss, cur, pin, pout, phi_f, hbuf, hist, ctl, blockIdx.x - 1);
 }
 #ifndef EHD_COUPLED_MIN_CTAS
 #define EHD_COUPLED_MIN_CTAS 7
@@ -871,7 +888,10 @@ __global__ void __launch_bounds__(128, EHD_COUPLED_MIN_CTAS) k_coupled<false>(KP
                                                            Ctl* ctl,
                                                            const double2* __restrict__ partials,
                                                            DevStats* stats) {
-  coupled_body<false>(k, ss, cur, pin, pout, phi_f, hbuf, hist, ctl, partials, stats, blockIdx.x);
+  if (blockIdx.x == 0)
+    coupled_keep(k, ss, cur, ctl, partials, stats);
+  else
+    coupled_body<false>(k, ss, cur, pin, pout, phi_f, hbuf, hist, ctl, blockIdx.x - 1);
 }
 #ifndef EHD_COUPLED16_MIN_CTAS
 #define EHD_COUPLED16_MIN_CTAS 6
@@ -885,7 +905,10 @@ __global__ void __launch_bounds__(128, EHD_COUPLED16_MIN_CTAS) k_coupled<true>(K
                                                             Ctl* ctl,
                                                             const double2* __restrict__ partials,
                                                             DevStats* stats) {
-  coupled_body<true>(k, ss, cur, pin, pout, phi_f, hbuf, hist, ctl, partials, stats, blockIdx.x);
+  if (blockIdx.x == 0)
+    coupled_keep(k, ss, cur, ctl, partials, stats);
+  else
+    coupled_body<true>(k, ss, cur, pin, pout, phi_f, hbuf, hist, ctl, blockIdx.x - 1);
 }
 
 // ------------------------------------------------------------------------------------
@@ -920,18 +943,36 @@ __global__ void __launch_bounds__(256) k_moments_batch(const StepSlot* __restric
                         S.tol, S.min_iter, S.max_iter, S.fixed_iter, w.y, S.mblocks);
 }
 
-// One form per storage precision, each over the work items of its slots: the FP32 form
-// has the register budget of the single-simulation FP32 pass (7 CTAs per SM), which a
-// kernel holding both forms could not have.
+// Slots of both storage precisions in one launch (seven droplets of 64^2 ... 512^2, alternately
+// FP32 and FP16: 25.5 us; in a launch for either 20.2 + 8.2 and the gap between them, 5 % of a
+// batch step).  6 CTAs per SM (80 registers), as the FP16 form; a batch of FP32 slots alone has
+// their own pass's 7.
 template <bool HALF>
-__global__ void __launch_bounds__(128, HALF ? 1 : EHD_COUPLED_MIN_CTAS)
-    k_coupled_batch(const StepSlot* __restrict__ slots, const int2* __restrict__ work,
-                    int cur) {
-  const int2 w = work[blockIdx.x];
-  const StepSlot& S = slots[w.x];
+__device__ __forceinline__ void coupled_slot(const StepSlot& S, int cur, int bid) {
   const Pops Pi = pops_copy(S.k, S.b, cur), Po = pops_copy(S.k, S.b, cur ^ 1);
-  coupled_body<HALF>(S.k, S.b.ss, cur, Pi, Po, S.b.phi, S.b.h, S.b.hist, S.b.ctl, S.b.partials,
-                     S.b.stats, w.y);
+  coupled_body<HALF>(S.k, S.b.ss, cur, Pi, Po, S.b.phi, S.b.h, S.b.hist, S.b.ctl, bid);
+}
+// The first nslots CTAs keep the slots' records.
+__device__ __forceinline__ void coupled_slot_keep(const StepSlot& S, int cur) {
+  coupled_keep(S.k, S.b.ss, cur, S.b.ctl, S.b.partials, S.b.stats);
+}
+__global__ void __launch_bounds__(128, EHD_COUPLED_MIN_CTAS)
+    k_coupled_batch(const StepSlot* __restrict__ slots, const int2* __restrict__ work, int cur,
+                    int nslots) {
+  if ((int)blockIdx.x < nslots) return coupled_slot_keep(slots[blockIdx.x], cur);
+  const int2 w = work[blockIdx.x - nslots];
+  coupled_slot<false>(slots[w.x], cur, w.y);
+}
+__global__ void __launch_bounds__(128, EHD_COUPLED16_MIN_CTAS)
+    k_coupled_batch_mixed(const StepSlot* __restrict__ slots, const int2* __restrict__ work,
+                          int cur, int nslots) {
+  if ((int)blockIdx.x < nslots) return coupled_slot_keep(slots[blockIdx.x], cur);
+  const int2 w = work[blockIdx.x - nslots];
+  const StepSlot& S = slots[w.x];
+  if (S.k.half)
+    coupled_slot<true>(S, cur, w.y);
+  else
+    coupled_slot<false>(S, cur, w.y);
 }
 
 // Diagnostics: puts the grid barrier's arrival count half the counter range behind every
@@ -1101,6 +1142,8 @@ __global__ void k_fields(KParams k, const StepState* __restrict__ ss, Pops pops,
 // Launchers
 // ------------------------------------------------------------------------------------
 static inline int blocks_for(int n, int t) { return (n + t - 1) / t; }
+// The coupled pass: one CTA that keeps the record, then one per 128 nodes.
+static inline int coupled_blocks(const KParams& kp) { return 1 + blocks_for(kp.nint, 128); }
 
 cudaError_t launch_step_set(const KParams& kp, const Buffers& b, int slot, long long n,
                             int first, cudaStream_t st) {
@@ -1152,10 +1195,10 @@ cudaError_t launch_moments(const KParams& kp, const Buffers& b, int cur, double 
 cudaError_t launch_coupled(const KParams& kp, const Buffers& b, int cur, cudaStream_t st) {
   const Pops Pi = pops_copy(kp, b, cur), Po = pops_copy(kp, b, cur ^ 1);
   if (kp.half)
-    k_coupled<true><<<blocks_for(kp.nint, 128), 128, 0, st>>>(kp, b.ss, cur, Pi, Po, b.phi, b.h,
+    k_coupled<true><<<coupled_blocks(kp), 128, 0, st>>>(kp, b.ss, cur, Pi, Po, b.phi, b.h,
                                                            b.hist, b.ctl, b.partials, b.stats);
   else
-    k_coupled<false><<<blocks_for(kp.nint, 128), 128, 0, st>>>(kp, b.ss, cur, Pi, Po, b.phi, b.h,
+    k_coupled<false><<<coupled_blocks(kp), 128, 0, st>>>(kp, b.ss, cur, Pi, Po, b.phi, b.h,
                                                             b.hist, b.ctl, b.partials, b.stats);
   return cudaGetLastError();
 }
@@ -1275,7 +1318,7 @@ cudaError_t add_coupled_node(cudaGraph_t g, const cudaGraphNode_t* deps, size_t 
   void* args[] = {&k, &ss, &cur, &pin, &pout, &phi, &h, &hist, &ctl, &partials, &stats};
   cudaKernelNodeParams p = {};
   p.func = kp.half ? (void*)k_coupled<true> : (void*)k_coupled<false>;
-  p.gridDim = dim3(blocks_for(kp.nint, 128));
+  p.gridDim = dim3(coupled_blocks(kp));
   p.blockDim = dim3(128);
   p.kernelParams = args;
   return cudaGraphAddKernelNode(out, g, deps, nd, &p);
@@ -1283,11 +1326,12 @@ cudaError_t add_coupled_node(cudaGraph_t g, const cudaGraphNode_t* deps, size_t 
 
 static cudaError_t add_batch_node(cudaGraph_t g, const cudaGraphNode_t* deps, size_t nd,
                                   cudaGraphNode_t* out, void* func, int threads,
-                                  const StepSlot* slots, const int2* work, int nwork, int cur) {
-  void* args[] = {&slots, &work, &cur};
+                                  const StepSlot* slots, const int2* work, int nwork, int cur,
+                                  int nslots = 0) {
+  void* args[] = {&slots, &work, &cur, &nslots};  // (the moments pass takes three)
   cudaKernelNodeParams p = {};
   p.func = func;
-  p.gridDim = dim3(nwork);
+  p.gridDim = dim3(nslots + nwork);
   p.blockDim = dim3(threads);
   p.kernelParams = args;
   return cudaGraphAddKernelNode(out, g, deps, nd, &p);
@@ -1301,10 +1345,10 @@ cudaError_t add_moments_batch_node(cudaGraph_t g, const cudaGraphNode_t* deps, s
 
 cudaError_t add_coupled_batch_node(cudaGraph_t g, const cudaGraphNode_t* deps, size_t nd,
                                    cudaGraphNode_t* out, const StepSlot* slots, const int2* work,
-                                   int nwork, int cur, bool half) {
+                                   int nwork, int nslots, int cur, bool half) {
   return add_batch_node(g, deps, nd, out,
-                        half ? (void*)k_coupled_batch<true> : (void*)k_coupled_batch<false>, 128,
-                        slots, work, nwork, cur);
+                        half ? (void*)k_coupled_batch_mixed : (void*)k_coupled_batch, 128,
+                        slots, work, nwork, cur, nslots);
 }
 
 cudaError_t add_poisson_node(cudaGraph_t g, cudaGraphNode_t* out, const KParams& kp,
