@@ -543,7 +543,8 @@ struct StepSlot {
 __host__ __device__ inline bool moments4_ok(const KParams& kp) {
   return !kp.slab && kp.N % 4 == 0 && kp.N == kp.nint;
 }
-__host__ __device__ inline int moments4_blocks(const KParams& kp) { return (kp.N / 4 + 255) / 256; }
+// CTAs of 256 threads at four nodes each
+__host__ __device__ inline int moments4_blocks(const KParams& kp) { return (kp.N + 1023) / 1024; }
 
 // Batched moments / coupled passes: one launch over work[] = (slot, block of that slot).
 cudaError_t add_moments_batch_node(cudaGraph_t g, const cudaGraphNode_t* deps, size_t nd,

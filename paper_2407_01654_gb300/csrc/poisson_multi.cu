@@ -469,7 +469,7 @@ bool multi_ok(const KParams& kp) {
 // they keep the front of the array, the loop's sums its end (the moments pass at 1024 x 2048 went
 // from 49.3 to 37.8 us without the tickets and the last CTA's reduction).
 bool multi_defers(const KParams& kp) {
-  return multi_ok(kp) && moments4_ok(kp) &&
+  return multi_ok(kp) &&
          moments4_blocks(kp) + (long long)multi_blocks(kp) * MULTI_D <= MAX_PARTIALS;
 }
 cudaError_t multi_prepare(const KParams& kp) {
