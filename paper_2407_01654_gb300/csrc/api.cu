@@ -274,7 +274,7 @@ int run_potential_loop(ehd_sim* s, int fixed, int max_iter) {
     }
     // the whole loop in one launch
     EHD_LAUNCH(s, 1, launch_poisson_resident(s->kp, rg, s->rthreads, s->rsmem, s->b,
-                                             s->stream));
+                                             fixed, s->stream));
     EHD_CUDA(cudaMemcpyAsync(s->h_ctl, s->b.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost,
                              s->stream));
     EHD_CUDA(cudaStreamSynchronize(s->stream));
@@ -605,21 +605,25 @@ int sim_create(const ehd_params* params, void* workspace, size_t workspace_bytes
       size_t sm;
       // whether the tiled loop of that many sub-iterations per exchange fits on chip
       auto fits = [&](int depth) {
-        const void* fk = nullptr;
         if (!resident_geometry(s->kp, sms, &g, &th, &sm, fixed_ty, depth) ||
-            (fk = resident_kernel(g.TY, depth, conv)) == nullptr ||
+            !resident_kernel(g.TY, depth, conv, false) ||
             2 * (size_t)g.ntx * g.nty * 8 * g.pmax > L.export_floats ||
-            (size_t)g.ntx * g.nty > L.rtiles ||
-            cudaFuncSetAttribute(fk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) !=
-                cudaSuccess)
+            (size_t)g.ntx * g.nty > L.rtiles)
           return false;
         int per_sm = 0;
+        for (int fixed = 0; fixed < 2; ++fixed) {  // the rule's form, a fixed count's
+          const void* fk = resident_kernel(g.TY, depth, conv, fixed != 0);
+          int n = 0;
+          if (cudaFuncSetAttribute(fk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) !=
+                  cudaSuccess ||
+              cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fk, th, sm) != cudaSuccess)
+            return false;
+          per_sm = fixed && per_sm < n ? per_sm : n;
+        }
         // the multi-step loops hold tensor memory for the whole launch: CTAs that share
         // an SM must fit its 512 columns together, or a CTA would wait in tcgen05.alloc
         // for one that only leaves at the end of the loop
         const int tcols = resident_tmem_columns(g.TY, depth);
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fk, th, sm) != cudaSuccess)
-          per_sm = 0;
         if (tcols < 0) per_sm = 0;
         if (tcols > 0 && per_sm > 512 / tcols) per_sm = 512 / tcols;
         return per_sm >= 1 && (long long)g.ntx * g.nty <= (long long)per_sm * sms;

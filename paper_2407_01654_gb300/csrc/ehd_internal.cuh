@@ -562,17 +562,18 @@ bool resident_geometry(const KParams& kp, int num_sms, ResidentGeom* g, int* thr
                        size_t* smem, int fixed_ty = 0, int depth = 0);
 // The single-simulation kernel of a tile height (nullptr if none): heights 8..64 in
 // steps of 8; with two sub-iterations per exchange, 24..64.
-const void* resident_kernel(int tile_rows, int depth = 0, bool conv = false);
+const void* resident_kernel(int tile_rows, int depth, bool conv, bool fixed);
 const void* resident_batch_kernel(int tile_rows);  // 16, 32 or 64; else nullptr
 // Tensor-memory columns (of the SM's 512) one CTA of that loop allocates: 0 for the
 // one-step loop, -1 for a shape with no kernel.
 int resident_tmem_columns(int tile_rows, int depth);
+// fixed: the solve's fixed count, or 0 under the rule.
 cudaError_t launch_poisson_resident(const KParams& kp, const ResidentGeom& g, int threads,
-                                    size_t smem, const Buffers& b, cudaStream_t st);
+                                    size_t smem, const Buffers& b, int fixed, cudaStream_t st);
 cudaError_t add_poisson_resident_node(cudaGraph_t graph, const cudaGraphNode_t* deps, size_t nd,
                                       cudaGraphNode_t* out, const KParams& kp,
                                       const ResidentGeom& g, int threads, size_t smem,
-                                      const Buffers& b);
+                                      const Buffers& b, int fixed);
 
 // Streaming with several sub-iterations per launch (poisson_multi.cu).
 constexpr long long MULTI_MIN_NODES = 600000;

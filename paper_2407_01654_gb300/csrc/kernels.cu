@@ -1437,7 +1437,8 @@ cudaError_t build_step_graph(const KParams& kp, const Buffers& b, int cur, doubl
     have = true;
     if ((e = record(1)) != cudaSuccess) return done(e);
     if (rg) {
-      if ((e = add_poisson_resident_node(g, &last, 1, &pn, kp, *rg, rthreads, rsmem, b)) !=
+      if ((e = add_poisson_resident_node(g, &last, 1, &pn, kp, *rg, rthreads, rsmem, b,
+                                         fixed_iter)) !=
           cudaSuccess)
         return done(e);
       last = pn;

@@ -54,6 +54,14 @@ __device__ __forceinline__ unsigned long long global_ns() {
 __device__ __forceinline__ void red_release_add(unsigned* p, unsigned v) {
   asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
+__device__ __forceinline__ unsigned atom_acq_rel_add(unsigned* p, unsigned v) {
+  unsigned old;
+  asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;"
+               : "=r"(old)
+               : "l"(p), "r"(v)
+               : "memory");
+  return old;
+}
 __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
   unsigned v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -617,7 +625,11 @@ __device__ __forceinline__ float gather_swapped(const float* sm, int i, int f, b
 
 }  // namespace
 
-template <int TY, bool CONV>
+// FIXED: a fixed count.  It needs no decision, so its last cycle ends with its last sub-iteration:
+// no second one where the count is odd, no band, no grid barrier and no collision to drop
+// (at K = 5 and 512 x 1024 21.8 us a solve against 29.0, at K = 2 and 256 x 256 8.3 against 10.3).
+// A kernel of its own, because the two endings in one spill registers at 56 rows and more.
+template <int TY, bool CONV, bool FIXED>
 __device__ __forceinline__ void resident_loop2(const KParams& k, const ResidentGeom& rg,
                                                float* __restrict__ hbuf,
                                                const float2* __restrict__ aq,
@@ -682,14 +694,14 @@ __device__ __forceinline__ void resident_loop2(const KParams& k, const ResidentG
   // sub-iteration, not converged
   const bool bad_state = __ldg(&ctl->nonfinite) != 0;
   const int min_iter = bad_state ? 1 : ctl->min_iter, max_iter = bad_state ? 1 : ctl->max_iter,
-            fixed = bad_state ? 0 : ctl->fixed_iter;
+            fixed = bad_state ? (FIXED ? 1 : 0) : ctl->fixed_iter;
   const float om = k.omega_h;
   constexpr int pstride = 8 * T::PMAX;
   const int warp = threadIdx.x >> 5;
   constexpr int dwarp = T::THREADS / 32 - 1;
 
   // TMEM for the parked state: warp w uses lanes 32 (w mod 4) .. + 31, columns 32 (w / 4)
-  if (warp == 0) {
+  if (!FIXED && warp == 0) {
     const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&s_taddr);
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst),
                  "n"(T::TCOLS)
@@ -723,7 +735,7 @@ __device__ __forceinline__ void resident_loop2(const KParams& k, const ResidentG
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t taddr = s_taddr + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(32 * (warp >> 2));
+  const uint32_t taddr = FIXED ? 0u : s_taddr + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(32 * (warp >> 2));
 
   // my ring node (thread r < number of ring nodes): frame index, flags, import source
   const int nring = 4 * (tw + 4) + 4 * th;
@@ -781,18 +793,21 @@ __device__ __forceinline__ void resident_loop2(const KParams& k, const ResidentG
   }
   __syncthreads();
 
+  const int cycles = (fixed + 1) / 2;
   unsigned target = 0;
   int cyc = 0, it = 0, conv = 0;
-  float rel = 0.0f;
+  float rel = 0.0f, num, den;
   int done = 0;
   for (;;) {
+    const bool last = FIXED && cyc + 1 >= cycles;
+    const bool sums1 = !FIXED || (last && (fixed & 1)), sums2 = !FIXED || last;  // wanted sums
     // ---- after the previous cycle's grid barrier: the deciding warp starts copying that
     // cycle's per-tile sums and the ring threads import the ring for this one.  Every
     // thread then collides, and the deciding warp applies the rule to the previous
     // cycle's two sub-iterations; the collision is dropped if the rule stopped the loop
     // (it writes shared memory only). ----
     if (cyc > 0) {
-      if (warp == dwarp) {
+      if (!FIXED && warp == dwarp) {
         // the previous cycle's sums of every tile (num and den of its two sub-iterations),
         // copied while the warp collides its nodes; lane l takes tiles l, l + 32, ...
         const float4* pp = reinterpret_cast<const float4*>(rpartials) + (size_t)((cyc - 1) & 1) * ntiles;
@@ -829,7 +844,7 @@ __device__ __forceinline__ void resident_loop2(const KParams& k, const ResidentG
         if (valid(2 * p + 1)) sm[i * T::PLANE + at0 + o1] = hs[i].y;
       }
     }
-    if (cyc > 0 && warp == dwarp) {
+    if (!FIXED && cyc > 0 && warp == dwarp) {
       // the rule, applied to the previous cycle's two sub-iterations in order
       cp_async_wait_all();
       const float4* pp = reinterpret_cast<const float4*>(rpartials) + (size_t)((cyc - 1) & 1) * ntiles;
@@ -901,9 +916,16 @@ __device__ __forceinline__ void resident_loop2(const KParams& k, const ResidentG
                                            : h_star(i, hr[i - 1], om, varphi, a, m1x, m1y, qs);
     }
     __syncthreads();  // post-collision populations and the rule's verdict visible
-    done = s_done;
+    if (!FIXED) done = s_done;
     if (done) break;
-    float num = 0.0f, den = 0.0f;
+    if (last && cyc == 0) {
+      // no grid barrier will have come before the write-back in place: this tile has read what
+      // it needs of its neighbours' state
+      target += ntiles;
+      if (threadIdx.x == 0) red_release_add(&ctl->bar_count, 1u);
+    }
+    num = 0.0f;
+    den = 0.0f;
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
       const int f0 = at0 + 2 * p * T::ROWS * PXF, f1 = at0 + (2 * p + 1) * T::ROWS * PXF;
@@ -921,15 +943,16 @@ __device__ __forceinline__ void resident_loop2(const KParams& k, const ResidentG
         }
       }
       const float2 d = __fadd2_rn(h_varphi2(h_sum8x2(h[p])), neg2(vold[p]));
-      if (valid(2 * p)) {
+      if (sums1 && valid(2 * p)) {
         num = __fmaf_rn(d.x, d.x, num);
         den = __fmaf_rn(vold[p].x, vold[p].x, den);
       }
-      if (valid(2 * p + 1)) {
+      if (sums1 && valid(2 * p + 1)) {
         num = __fmaf_rn(d.y, d.y, num);
         den = __fmaf_rn(vold[p].y, vold[p].y, den);
       }
     }
+    if (last && (fixed & 1)) break;
     if (rlayer1) {
 #pragma unroll
       for (int i = 1; i < 9; ++i)
@@ -937,13 +960,15 @@ __device__ __forceinline__ void resident_loop2(const KParams& k, const ResidentG
     }
     // park the state after the first sub-iteration in TMEM (restored if the rule stops
     // the loop there)
-    tmem_store32(taddr, h);
+    if (!FIXED) tmem_store32(taddr, h);
+    if (!FIXED) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      num += __shfl_xor_sync(0xffffffffu, num, o);
-      den += __shfl_xor_sync(0xffffffffu, den, o);
+      for (int o = 16; o > 0; o >>= 1) {
+        num += __shfl_xor_sync(0xffffffffu, num, o);
+        den += __shfl_xor_sync(0xffffffffu, den, o);
+      }
+      if ((threadIdx.x & 31) == 0) s_w1[warp] = make_float2(num, den);
     }
-    if ((threadIdx.x & 31) == 0) s_w1[warp] = make_float2(num, den);
     // ---- sub-iteration 2: collide tile and inner ring, stream into the tile.  Direction
     // i of the node at x goes to slot opp(i) of the cell at x + c_i, the one slot the
     // thread of node x itself read in the first streaming, so no thread can still be
@@ -985,7 +1010,7 @@ __device__ __forceinline__ void resident_loop2(const KParams& k, const ResidentG
                  : h_star(i, hr[i - 1], om, varphi, a, m1x, m1y, qs);
     }
     __syncthreads();
-    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    if (!FIXED) asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     num = 0.0f;
     den = 0.0f;
 #pragma unroll
@@ -1005,21 +1030,24 @@ __device__ __forceinline__ void resident_loop2(const KParams& k, const ResidentG
         }
       }
       const float2 d = __fadd2_rn(h_varphi2(h_sum8x2(h[p])), neg2(vold[p]));
-      if (valid(2 * p)) {
+      if (sums2 && valid(2 * p)) {
         num = __fmaf_rn(d.x, d.x, num);
         den = __fmaf_rn(vold[p].x, vold[p].x, den);
       }
-      if (valid(2 * p + 1)) {
+      if (sums2 && valid(2 * p + 1)) {
         num = __fmaf_rn(d.y, d.y, num);
         den = __fmaf_rn(vold[p].y, vold[p].y, den);
       }
     }
+    if (last) break;
+    if (!FIXED) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      num += __shfl_xor_sync(0xffffffffu, num, o);
-      den += __shfl_xor_sync(0xffffffffu, den, o);
+      for (int o = 16; o > 0; o >>= 1) {
+        num += __shfl_xor_sync(0xffffffffu, num, o);
+        den += __shfl_xor_sync(0xffffffffu, den, o);
+      }
+      if ((threadIdx.x & 31) == 0) s_w2[warp] = make_float2(num, den);
     }
-    if ((threadIdx.x & 31) == 0) s_w2[warp] = make_float2(num, den);
     {
       // export band: the new state of the tile's two outer rows and columns, gathered
       // again from the second sub-iteration's post-collision populations (still in
@@ -1042,20 +1070,23 @@ __device__ __forceinline__ void resident_loop2(const KParams& k, const ResidentG
     __syncthreads();
     target += ntiles;
     if (threadIdx.x < 32) {
-      constexpr int nwarps = T::THREADS / 32;
+      constexpr int nwarps = FIXED ? 0 : T::THREADS / 32;
       const bool in = (int)threadIdx.x < nwarps;
       float2 v1 = in ? s_w1[threadIdx.x] : make_float2(0.0f, 0.0f);
       float2 v2 = in ? s_w2[threadIdx.x] : make_float2(0.0f, 0.0f);
+      if (!FIXED) {
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        v1.x += __shfl_xor_sync(0xffffffffu, v1.x, o);
-        v1.y += __shfl_xor_sync(0xffffffffu, v1.y, o);
-        v2.x += __shfl_xor_sync(0xffffffffu, v2.x, o);
-        v2.y += __shfl_xor_sync(0xffffffffu, v2.y, o);
+        for (int o = 16; o > 0; o >>= 1) {
+          v1.x += __shfl_xor_sync(0xffffffffu, v1.x, o);
+          v1.y += __shfl_xor_sync(0xffffffffu, v1.y, o);
+          v2.x += __shfl_xor_sync(0xffffffffu, v2.x, o);
+          v2.y += __shfl_xor_sync(0xffffffffu, v2.y, o);
+        }
       }
       if (threadIdx.x == 0) {
-        reinterpret_cast<float4*>(rpartials)[(size_t)(cyc & 1) * ntiles + tile] =
-            make_float4(v1.x, v1.y, v2.x, v2.y);
+        if (!FIXED)
+          reinterpret_cast<float4*>(rpartials)[(size_t)(cyc & 1) * ntiles + tile] =
+              make_float4(v1.x, v1.y, v2.x, v2.y);
         int ok = 1;
         red_release_add(&ctl->bar_count, 1u);
         const unsigned long long t0 = global_ns();
@@ -1073,7 +1104,7 @@ __device__ __forceinline__ void resident_loop2(const KParams& k, const ResidentG
     if (!s_ok) {
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncthreads();
-      if (warp == 0) {
+      if (!FIXED && warp == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_taddr),
                      "n"(T::TCOLS)
@@ -1083,17 +1114,80 @@ __device__ __forceinline__ void resident_loop2(const KParams& k, const ResidentG
     }
     ++cyc;
   }
-  if (done == 1) tmem_load32(taddr, h);  // the loop stopped after the first sub-iteration
+  if (!FIXED && done == 1) tmem_load32(taddr, h);  // the loop stopped after the first sub-iteration
+
+  if (FIXED) {
+    // The last sub-iteration's sums, a statistic here: every tile leaves its own and goes on to
+    // its write-back; the last one to do so adds them in the order of the rule.
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      num += __shfl_xor_sync(0xffffffffu, num, o);
+      den += __shfl_xor_sync(0xffffffffu, den, o);
+    }
+    if ((threadIdx.x & 31) == 0) s_w1[warp] = make_float2(num, den);
+    if (threadIdx.x == 0) {
+      int ok = 1;
+      const unsigned long long t0 = global_ns();
+      // (only a single cycle's early arrivals can be outstanding)
+      while ((int)(ld_acquire(&ctl->bar_count) - target) < 0) {
+        if (global_ns() - t0 > BARRIER_TIMEOUT_NS) {
+          atomicOr(&ctl->bar_error, 1);
+          ok = 0;
+          break;
+        }
+      }
+      s_ok = ok;
+    }
+    __syncthreads();
+    if (s_ok && warp == 0) {
+      constexpr int nwarps = T::THREADS / 32;
+      const int lane = threadIdx.x;
+      float2 v = lane < nwarps ? s_w1[lane] : make_float2(0.0f, 0.0f);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+        v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+      }
+      int all = 0;
+      if (lane == 0) {
+        rpartials[tile] = v;
+        all = atom_acq_rel_add(&ctl->bar_count, 1u) == target + (unsigned)ntiles - 1u;
+      }
+      if (__shfl_sync(0xffffffffu, all, 0)) {
+        float a = 0.0f, b = 0.0f;
+        for (int t = lane; t < ntiles; t += 32) {
+          const float2 w = __ldcg(rpartials + t);
+          a += w.x;
+          b += w.y;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          a += __shfl_xor_sync(0xffffffffu, a, o);
+          b += __shfl_xor_sync(0xffffffffu, b, o);
+        }
+        if (lane == 0) {
+          ctl->iter = fixed;
+          const float r = a == 0.0f && b == 0.0f ? 0.0f
+                          : b == 0.0f            ? __int_as_float(0x7f800000)
+                                                 : sqrtf(a / b);
+          ctl->rel = (double)r;
+          ctl->converged = bad_state ? (double)r < tol : 1;
+          ctl->done = 1;
+        }
+      }
+    }
+    done = s_ok ? 0 : -1;
+  }
 
   // the registers hold the final state: write it back in place
 #pragma unroll
   for (int s = 0; s < NPT; ++s) {
-    if (!valid(s)) continue;
+    if (!valid(s) || done < 0) continue;
     const int g = (int)EHD_IDX(k, (ty0 + ly0 + s * T::ROWS) * nx + tx0 + lx, N);
 #pragma unroll
     for (int i = 0; i < 8; ++i) hsrc[i * N + g] = (s & 1) ? h[s >> 1][i].y : h[s >> 1][i].x;
   }
-  if (tile == 0 && (int)threadIdx.x == dwarp * 32) {
+  if (!FIXED && tile == 0 && (int)threadIdx.x == dwarp * 32) {
     ctl->iter = it;
     ctl->rel = (double)rel;
     ctl->converged = conv;
@@ -1101,7 +1195,7 @@ __device__ __forceinline__ void resident_loop2(const KParams& k, const ResidentG
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (warp == 0) {
+  if (!FIXED && warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(s_taddr),
                  "n"(T::TCOLS)
@@ -1109,12 +1203,12 @@ __device__ __forceinline__ void resident_loop2(const KParams& k, const ResidentG
   }
 }
 
-template <int TY, bool CONV>
+template <int TY, bool CONV, bool FIXED>
 __global__ void __launch_bounds__(Tile2<TY>::THREADS, 1)
     k_poisson_resident2(KParams k, ResidentGeom rg, float* __restrict__ hbuf,
                         const float2* __restrict__ aq, float* __restrict__ exports,
                         float2* __restrict__ rpartials, Ctl* ctl) {
-  resident_loop2<TY, CONV>(k, rg, hbuf, aq, exports, rpartials, ctl, blockIdx.x, gridDim.x);
+  resident_loop2<TY, CONV, FIXED>(k, rg, hbuf, aq, exports, rpartials, ctl, blockIdx.x, gridDim.x);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1703,18 +1797,23 @@ __global__ void __launch_bounds__(TileD<TY, 3>::THREADS, 1)
 }
 
 // The kernel of a tile height, sub-iterations per exchange (0: the one-step loop;
-// 2: heights 24 to 64; 3: heights 48 to 64) and potential scheme (conv: the conventional
+// 2: heights 24 to 64, the form for a fixed count where asked; 3: heights 48 to 64) and potential scheme (conv: the conventional
 // one, on the one- and two-step loops), or nullptr.
 template <bool CONV>
-const void* resident_kernel_of(int ty, int depth) {
+const void* resident_kernel_of(int ty, int depth, bool fixed) {
   if (depth == 2) {
+    auto of = [&](auto t) {
+      constexpr int TY = decltype(t)::value;
+      return fixed ? (const void*)k_poisson_resident2<TY, CONV, true>
+                   : (const void*)k_poisson_resident2<TY, CONV, false>;
+    };
     switch (ty) {
-      case 24: return (const void*)k_poisson_resident2<24, CONV>;
-      case 32: return (const void*)k_poisson_resident2<32, CONV>;
-      case 40: return (const void*)k_poisson_resident2<40, CONV>;
-      case 48: return (const void*)k_poisson_resident2<48, CONV>;
-      case 56: return (const void*)k_poisson_resident2<56, CONV>;
-      case 64: return (const void*)k_poisson_resident2<64, CONV>;
+      case 24: return of(std::integral_constant<int, 24>{});
+      case 32: return of(std::integral_constant<int, 32>{});
+      case 40: return of(std::integral_constant<int, 40>{});
+      case 48: return of(std::integral_constant<int, 48>{});
+      case 56: return of(std::integral_constant<int, 56>{});
+      case 64: return of(std::integral_constant<int, 64>{});
       default: return nullptr;
     }
   }
@@ -1740,15 +1839,16 @@ const void* resident_kernel_of(int ty, int depth) {
     default: return nullptr;
   }
 }
-const void* resident_kernel(int ty, int depth, bool conv) {
-  return conv ? resident_kernel_of<true>(ty, depth) : resident_kernel_of<false>(ty, depth);
+const void* resident_kernel(int ty, int depth, bool conv, bool fixed) {
+  return conv ? resident_kernel_of<true>(ty, depth, fixed)
+              : resident_kernel_of<false>(ty, depth, fixed);
 }
 
 // Tensor-memory columns one CTA of the multi-step loop allocates (tcgen05.alloc; 0 for
 // the one-step loop, which parks nothing), or -1 for a shape with no kernel.
 int resident_tmem_columns(int ty, int depth) {
   if (depth == 0) return 0;
-  if (!resident_kernel(ty, depth, false)) return -1;
+  if (!resident_kernel(ty, depth, false, false)) return -1;
   switch (depth == 2 ? ty : 1000 + ty) {
     case 24: return Tile2<24>::TCOLS;
     case 32: return Tile2<32>::TCOLS;
@@ -1832,9 +1932,9 @@ bool resident_geometry(const KParams& kp, int num_sms, ResidentGeom* g, int* thr
 }
 
 cudaError_t launch_poisson_resident(const KParams& kp, const ResidentGeom& g, int threads,
-                                    size_t smem, const Buffers& b, cudaStream_t st) {
+                                    size_t smem, const Buffers& b, int fixed, cudaStream_t st) {
   if (g.cluster.size > 0) return launch_poisson_cluster(kp, g, b, st);
-  const void* f = resident_kernel(g.TY, g.depth, kp.scheme == 1);
+  const void* f = resident_kernel(g.TY, g.depth, kp.scheme == 1, fixed > 0);
   if (!f) return cudaErrorInvalidValue;
   KParams k = kp;
   ResidentGeom gg = g;
@@ -1850,9 +1950,9 @@ cudaError_t launch_poisson_resident(const KParams& kp, const ResidentGeom& g, in
 cudaError_t add_poisson_resident_node(cudaGraph_t graph, const cudaGraphNode_t* deps, size_t nd,
                                       cudaGraphNode_t* out, const KParams& kp,
                                       const ResidentGeom& g, int threads, size_t smem,
-                                      const Buffers& b) {
+                                      const Buffers& b, int fixed) {
   if (g.cluster.size > 0) return add_poisson_cluster_node(graph, deps, nd, out, kp, g, b);
-  const void* f = resident_kernel(g.TY, g.depth, kp.scheme == 1);
+  const void* f = resident_kernel(g.TY, g.depth, kp.scheme == 1, fixed > 0);
   if (!f) return cudaErrorInvalidValue;
   KParams k = kp;
   ResidentGeom gg = g;
