@@ -648,15 +648,14 @@ int sim_create(const ehd_params* params, void* workspace, size_t workspace_bytes
             }
         // and the other lattices run two sub-iterations per exchange where that fits the same
         // tiles, whose sums and so decisions are the one-step loop's bit for bit.  Per step at
-        // K = 2 and 5 it takes 23.9 and 32.8 us against 28.0 and 39.1 at 256 x 256, 49.8 and 63.1
-        // against 51.3 and 63.8 at 512 x 1024.  A cycle makes two sub-iterations whether the
-        // second is wanted or not: with tiles above 32 rows a fixed count of 1 (37.2 against
-        // 35.9 us at 512 x 700), with 48 and more also one of 3 (56.6 against 55.4 at
-        // 512 x 1024), stays with the one-step loop.
+        // K = 2 and 5 it took 23.9 and 32.8 us against 28.0 and 39.1 at 256 x 256, before a
+        // fixed count had its own ending; with it a solve of K = 3 at 512 x 1024 takes 16.2 us
+        // against 21.8 (14.6 at 512 x 800, tiles of 48 rows).
+        // A fixed count of 1 exchanges nothing either way: with tiles above 32 rows it stays
+        // with the one-step loop.
         const ResidentGeom one = g;
-        const int k = params->poisson_fixed_iter;
         if (params->poisson_loop == EHD_LOOP_AUTO && fixed_ty == 0 && s->rg.cluster.size == 0 &&
-            !(one.TY > 32 && k == 1) && !(one.TY >= 48 && k == 3) && fits(2) && g.TY == one.TY &&
+            !(one.TY > 32 && params->poisson_fixed_iter == 1) && fits(2) && g.TY == one.TY &&
             g.nty == one.nty)
           take();
       }
