@@ -245,6 +245,12 @@ int ehd_solve_potential(ehd_sim* sim, double tol, int max_iter, int* iters,
  * Errors: EHD_ERR_INVALID_ARG (null pointer, a bit beyond EHD_F_MU, bad mem). */
 int ehd_read_fields(ehd_sim* sim, unsigned mask, void* const* out, int mem);
 
+/* Diagnostics: 1 if ehd_read_fields(..., EHD_DEVICE) writes n arrays of `bytes` bytes at
+ * these addresses straight from its kernel, 0 if it goes through copies that the runtime
+ * checks: memory of another kind or device, misaligned, not whole inside its allocation, or
+ * overlapping one another.  Touches none of the memory. */
+int ehd_diag_direct_outputs(void* const* out, int n, size_t bytes);
+
 /* The contact line of a drop sitting on the bottom wall, from the current populations
  * (the normalised contact-radius histories of Sec. 7.2, Fig. 11, are radius / its initial
  * value): on each of the first two lattice rows the crossings of phi = level are placed

@@ -1,4 +1,6 @@
 // Host side of the C ABI declared in include/ehd.h.
+#include <cuda.h>
+
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -452,20 +454,52 @@ int stage_in(ehd_sim* s, const void* src, int slot, int mem) {
   return EHD_OK;
 }
 
-// Whether a kernel on the current device may write float32 arrays at these addresses: device
-// memory of this device, 4-byte aligned.  (What else a caller calls a device array goes through
-// a copy, which reports what it cannot reach.)
-bool writable_here(void* const* out, int n) {
+// The bounds of the device allocation that holds p; false where the driver cannot tell.
+bool allocation_of(const void* p, uintptr_t* base, size_t* size) {
+  using Range = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+  static const Range range = [] {  // from the driver that is loaded: the library links none
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault,
+                                         &found) != cudaSuccess ||
+        found != cudaDriverEntryPointSuccess)
+      f = nullptr;
+    cudaGetLastError();
+    return reinterpret_cast<Range>(f);
+  }();
+  CUdeviceptr b = 0;
+  if (!range || range(&b, size, reinterpret_cast<CUdeviceptr>(p)) != CUDA_SUCCESS) return false;
+  *base = (uintptr_t)b;
+  return true;
+}
+
+// Whether a kernel on the current device may write n arrays of `bytes` bytes of float32 at
+// these addresses: device memory of this device, 4-byte aligned, every array whole inside its
+// allocation and apart from the others.  What else a caller calls a device array goes through
+// copies, one field after the other, which the runtime checks before anything is written.
+bool writable_here(void* const* out, int n, size_t bytes) {
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  if (cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
   for (int j = 0; j < n; ++j) {
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, out[j]) != cudaSuccess) {
       cudaGetLastError();
       return false;
     }
-    if (a.type != cudaMemoryTypeDevice || a.device != dev || (reinterpret_cast<uintptr_t>(out[j]) & 3u))
+    const uintptr_t p = reinterpret_cast<uintptr_t>(out[j]);
+    if (a.type != cudaMemoryTypeDevice || a.device != dev || (p & 3u)) return false;
+    uintptr_t base = 0;
+    size_t size = 0;
+    if (!allocation_of(out[j], &base, &size) || p < base || bytes > size ||
+        p - base > size - bytes)
       return false;
+    for (int i = 0; i < j; ++i) {
+      const uintptr_t o = reinterpret_cast<uintptr_t>(out[i]);
+      if ((p > o ? p - o : o - p) < bytes) return false;
+    }
   }
   return true;
 }
@@ -956,6 +990,13 @@ int ehd_read_stats(ehd_sim* s, ehd_stats* out) {
   return st;
 }
 
+int ehd_diag_direct_outputs(void* const* out, int n, size_t bytes) {
+  if (!out || n < 1 || n > EHD_NUM_FIELDS) return 0;
+  for (int j = 0; j < n; ++j)
+    if (!out[j]) return 0;
+  return writable_here(out, n, bytes) ? 1 : 0;
+}
+
 int ehd_read_fields(ehd_sim* s, unsigned mask, void* const* out, int mem) {
   NvtxRange range("ehd_read_fields");
   if (!s || !out || (mem != EHD_HOST && mem != EHD_DEVICE) || (mask & ~((1u << EHD_NUM_FIELDS) - 1u)))
@@ -968,7 +1009,7 @@ int ehd_read_fields(ehd_sim* s, unsigned mask, void* const* out, int mem) {
       ++nf;
     }
   const size_t N = (size_t)s->kp.N;
-  if (mem == EHD_DEVICE && writable_here(out, nf)) {
+  if (mem == EHD_DEVICE && writable_here(out, nf, N * sizeof(float))) {
     // straight into the caller's arrays
     float* outs[EHD_NUM_FIELDS];
     for (int j = 0; j < nf; ++j) outs[j] = static_cast<float*>(out[j]);

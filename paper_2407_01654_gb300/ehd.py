@@ -126,6 +126,8 @@ SIGNATURES = {
                                            ctypes.POINTER(ctypes.c_double)]),
     "ehd_read_fields": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_uint,
                                        ctypes.POINTER(ctypes.c_void_p), ctypes.c_int]),
+    "ehd_diag_direct_outputs": (ctypes.c_int, [ctypes.POINTER(ctypes.c_void_p), ctypes.c_int,
+                                               ctypes.c_size_t]),
     "ehd_contact_line": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_double,
                                         ctypes.POINTER(ctypes.c_double)]),
     "ehd_diag_index_errors": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ctypes.c_uint)]),
