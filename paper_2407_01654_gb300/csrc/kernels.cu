@@ -164,6 +164,26 @@ __device__ __forceinline__ float warp_sum(float v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
+// The warp sums of a[0], b[0], a[1], b[1], ... in lanes 0, 4, 8, ...: warp_sum's tree for each of
+// the eight, in 9 shuffles instead of 40, because at each level a half of the lanes carries on a
+// half of the values.
+__device__ __forceinline__ float warp_sum8(const float (&a)[4], const float (&b)[4], int lane) {
+  float v[8];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    v[2 * j] = a[j];
+    v[2 * j + 1] = b[j];
+  }
+#pragma unroll
+  for (int o = 16, n = 4; o > 2; o >>= 1, n >>= 1) {
+    const bool hi = (lane & o) != 0;
+#pragma unroll
+    for (int j = 0; j < n; ++j)
+      v[j] = (hi ? v[j + n] : v[j]) + __shfl_xor_sync(0xffffffffu, hi ? v[j] : v[j + n], o);
+  }
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
 
 }  // namespace
 
@@ -343,32 +363,40 @@ __device__ __forceinline__ void moments_tail(const KParams& k, const StepState* 
 // The moments pass without the cross-CTA reduction (an on-chip potential loop without a
 // neutralised source needs neither the mean charge nor the sums before it runs): each CTA
 // leaves its FP64 partial, the coupled pass reduces them for the statistics, and block 0
-// sets the loop control.  (A non-finite flag is applied by the loop itself.)
+// sets the loop control.  (A non-finite flag is applied by the loop itself.)  A thread brings G
+// values of each sum, which are added to its warp's others of the same index in FP32 and to one
+// another in FP64.
+template <int G>
 __device__ __forceinline__ void moments_partial_only(const KParams& k,
                                                      const StepState* __restrict__ ss,
                                                      double2* __restrict__ partials, Ctl* ctl,
                                                      double tol, int min_iter, int max_iter,
                                                      int fixed_iter, int bid, int nblk,
-                                                     float phi_acc, float q_acc, int bad) {
-  __shared__ float2 s_sum[8];
-  const float wp = warp_sum(phi_acc), wq = warp_sum(q_acc);
+                                                     const float (&phi)[G], const float (&q)[G],
+                                                     int bad) {
+  __shared__ float s_sum[2][8 * G];  // phi's, q's: [index][warp], 8 warps a CTA
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) s_sum[warp] = make_float2(wp, wq);
+  if constexpr (G == 1) {
+    const float wp = warp_sum(phi[0]), wq = warp_sum(q[0]);
+    if (lane == 0) {
+      s_sum[0][warp] = wp;
+      s_sum[1][warp] = wq;
+    }
+  } else {
+    const float w = warp_sum8(phi, q, lane);
+    if ((lane & 3) == 0) s_sum[(lane >> 2) & 1][8 * (lane >> 3) + warp] = w;
+  }
   if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(&ctl->nonfinite, 1);
   __syncthreads();
   if (warp != 0) return;
-  const int nw = (int)(blockDim.x >> 5);
-  double a = 0.0, b = 0.0;
-  if (lane < nw) {
-    a = (double)s_sum[lane].x;
-    b = (double)s_sum[lane].y;
-  }
+  // a fixed FP64 tree, phi's on the low lanes and q's on the high ones (FP64 additions are slow:
+  // five of them instead of ten for 32 pairs)
+  const float* e = s_sum[lane >> 4] + (lane & 15);
+  double a = (lane & 15) < 8 * G ? (double)e[0] : 0.0;
+  if constexpr (G == 4) a += (double)e[16];
 #pragma unroll
-  for (int o = 4; o > 0; o >>= 1) {  // the same fixed tree as moments_tail
-    a += __shfl_xor_sync(0xffffffffu, a, o);
-    b += __shfl_xor_sync(0xffffffffu, b, o);
-  }
-  if (lane == 0) partials[bid] = make_double2(a, b);
+  for (int o = G == 1 ? 4 : 8; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  if ((lane & 15) == 0) reinterpret_cast<double*>(partials + bid)[lane >> 4] = a;
   if (bid == 0 && lane == 0) {
     ctl->iter = 0;
     ctl->done = 0;
@@ -480,8 +508,8 @@ __device__ __forceinline__ void moments4_body(const KParams& k, const StepState*
     moments_tail(k, ss, partials, ctl, tol, min_iter, max_iter, fixed_iter, bid, nblk, phi_acc,
                  q_acc, bad);
   else
-    moments_partial_only(k, ss, partials, ctl, tol, min_iter, max_iter, fixed_iter, bid, nblk,
-                         phi_acc, q_acc, bad);
+    moments_partial_only<1>(k, ss, partials, ctl, tol, min_iter, max_iter, fixed_iter, bid, nblk,
+                            {phi_acc}, {q_acc}, bad);
 }
 template <bool TAIL, bool HALF>
 __global__ void __launch_bounds__(256) k_moments4(KParams k, const StepState* __restrict__ ss,
@@ -519,22 +547,20 @@ __global__ void __launch_bounds__(256) k_moments_odd(KParams k, const StepState*
     lo[c] = ld_g0_lo<HALF>(k, pops, idx);
     R[c] = __ldg(hist + 3 * (size_t)k.N + idx);
   }
-  float phi_acc = 0.0f, q_acc = 0.0f;
+  float phi[4] = {}, q[4] = {};
   int bad = 0;
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
     const int idx = first + 256 * c;
     if (idx >= k.N) break;
-    float phi, q;
-    moments_of(g[c], lo[c], l[c], R[c], phi, q);
-    phi_out[idx] = phi;
-    aq[idx] = make_float2(potential_coef(k, phi), q);
-    bad |= !(isfinite(phi) && isfinite(q));
-    phi_acc += phi;
-    q_acc += q;
+    moments_of(g[c], lo[c], l[c], R[c], phi[c], q[c]);
+    phi_out[idx] = phi[c];
+    aq[idx] = make_float2(potential_coef(k, phi[c]), q[c]);
+    bad |= !(isfinite(phi[c]) && isfinite(q[c]));
   }
-  moments_partial_only(k, ss, partials, ctl, tol, min_iter, max_iter, fixed_iter, blockIdx.x,
-                       gridDim.x, phi_acc, q_acc, bad);
+  // the sums stay FP32 over 32 consecutive nodes and FP64 beyond, as k_moments forms them
+  moments_partial_only<4>(k, ss, partials, ctl, tol, min_iter, max_iter, fixed_iter, blockIdx.x,
+                          gridDim.x, phi, q, bad);
 }
 // The moments pass of a lattice and its grid: four nodes per thread, with the cross-CTA tail or
 // (deferred; no slab) without; a node count that is no multiple of 4, or a slab, one node at a
