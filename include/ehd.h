@@ -57,7 +57,8 @@ enum { EHD_FP32 = 0, EHD_FP16DEV = 1 };
  * with the populations held on chip (only for lattices that fit, about 600k nodes on a
  * GB300; with the library's own tiles, lattices up to about 46k nodes run on one
  * thread-block cluster); AUTO picks RESIDENT where it fits, RESIDENT2 where that fits the
- * same tiles beyond one cluster. */
+ * same tiles beyond one cluster, and under the stopping rule on tiles above 32 rows the one of
+ * the two that the counts of the steps so far ask for. */
 enum {
   EHD_LOOP_AUTO = 0,
   EHD_LOOP_STREAM = 1,
@@ -221,7 +222,8 @@ int ehd_use_graphs(ehd_sim* sim, int enable);
 
 
 /* Which potential loop this simulation runs: EHD_LOOP_STREAM, EHD_LOOP_RESIDENT,
- * EHD_LOOP_RESIDENT2 or EHD_LOOP_RESIDENT3 (negative: invalid handle). */
+ * EHD_LOOP_RESIDENT2 or EHD_LOOP_RESIDENT3 (negative: invalid handle).  With EHD_LOOP_AUTO
+ * it can change between two calls of ehd_step. */
 int ehd_loop_kind(const ehd_sim* sim);
 
 /* Statistics accumulated since they were last cleared (by ehd_step with stats, or by this

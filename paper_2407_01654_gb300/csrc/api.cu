@@ -6,6 +6,7 @@
 #include <cstring>
 #include <new>
 #include <thread>
+#include <utility>
 #include <vector>
 
 #include "../../include/ehd.h"
@@ -321,7 +322,7 @@ int run_potential_loop(ehd_sim* s, int fixed, int max_iter) {
   }
 }
 
-void destroy_graphs(ehd_sim* s) {
+void destroy_graphs(LoopForm* s) {
   for (int c = 0; c < 2; ++c) {
     if (s->exec[c]) cudaGraphExecDestroy(s->exec[c]);
     if (s->graph[c]) cudaGraphDestroy(s->graph[c]);
@@ -336,6 +337,14 @@ void destroy_graphs(ehd_sim* s) {
   s->mgraphs_ok = false;
   s->pgraphs_ok = false;
   s->pgraphs_tried = false;
+}
+
+// Every graph of the simulation, to be built again when it is next wanted.
+void forget_graphs(ehd_sim* s) {
+  for (LoopForm* f : {static_cast<LoopForm*>(s), &s->other}) {
+    destroy_graphs(f);
+    f->graphs_tried = false;
+  }
 }
 
 // The profiling form of the step graphs: event-record nodes before the moments pass and
@@ -405,6 +414,54 @@ void ensure_graphs(ehd_sim* s) {
     }
   }
   s->mgraphs_ok = mok;
+}
+
+// Under the rule a cycle of the two-step loop makes two sub-iterations whether the second is
+// wanted or not, which on tall tiles costs more than the exchange it saves where the solve
+// takes one, and on the tallest where it takes three.  A step with the one- and the two-step
+// loop in us, by rows of a tile (lattice):
+//   K = 1   32 (512 x 512) 29.8, 29.6;  40 (512 x 700) 36.2, 37.5;  48 (512 x 800) 40.0, 41.5;
+//           56 (512 x 1024) 47.4, 50.1
+//   K = 3   40 44.5, 43.0;  48 47.9, 47.4;  56 55.8, 57.5
+//   K = 2, 4, 5, 7 up to 56 rows: the two-step loop is the faster one or equal
+// (On 64 rows, 576 x 1024, the rule's two-step loop is the slower one at every count, 62.4
+// against 54.2 at K = 1, 80.7 against 72.0 at K = 5, 149.5 against 142.6 at K = 21: it is not
+// taken there at all.)
+bool one_step_wins(int rows, int k) { return rows > 32 && (k == 1 || (k == 3 && rows >= 56)); }
+
+void swap_forms(ehd_sim* s) { std::swap(static_cast<LoopForm&>(*s), s->other); }
+
+// The two-step loop, before the count of the new state's solves is known.
+void first_form(ehd_sim* s) {
+  if (!s->two_forms) return;
+  if (s->rg.depth != 2) swap_forms(s);
+  s->form_steps = 0;
+  s->want_one = false;
+  s->h_ctl[1].iter = 0;
+}
+
+// After `steps` steps run as graphs: every 256 steps the device is asked for the count of its
+// last solve, the answer read 256 steps (or more, where the host runs ahead) later, so that
+// nothing waits.  Two answers in a row that ask for the other loop change over to it; the
+// states and decisions of the two are the same bit for bit.
+int follow_count(ehd_sim* s, int steps) {
+  constexpr int EVERY = 256;
+  if (!s->two_forms || (s->form_steps += steps) < EVERY) return EHD_OK;
+  s->form_steps = 0;
+  const int k = *static_cast<volatile int*>(&s->h_ctl[1].iter);
+  const bool want_one = one_step_wins(s->rg.TY, k);
+  if (want_one == s->want_one && want_one != (s->rg.depth == 0)) {
+    swap_forms(s);
+    ensure_graphs(s);
+    if (!s->graphs_ok) {
+      swap_forms(s);
+      s->two_forms = false;
+    }
+  }
+  s->want_one = want_one;
+  EHD_CUDA(cudaMemcpyAsync(&s->h_ctl[1].iter, &s->b.ctl->iter, sizeof(int),
+                           cudaMemcpyDeviceToHost, s->stream));
+  return EHD_OK;
 }
 
 // dst[j][i] = (To)src[j][i] for j < nf, i < n: the conversions between the caller's
@@ -681,17 +738,23 @@ int sim_create(const ehd_params* params, void* workspace, size_t workspace_bytes
               break;
             }
         // and the other lattices run two sub-iterations per exchange where that fits the same
-        // tiles, whose sums and so decisions are the one-step loop's bit for bit.  Per step at
-        // K = 2 and 5 it took 23.9 and 32.8 us against 28.0 and 39.1 at 256 x 256, before a
-        // fixed count had its own ending; with it a solve of K = 3 at 512 x 1024 takes 16.2 us
-        // against 21.8 (14.6 at 512 x 800, tiles of 48 rows).
+        // tiles, whose sums and so decisions are the one-step loop's bit for bit: 3.77 -> 2.27 us
+        // per sub-iteration at 256 x 256 under the rule; a fixed count, which has an ending of
+        // its own, takes 16.2 us a solve at K = 3 and 512 x 1024 against 21.8.
         // A fixed count of 1 exchanges nothing either way: with tiles above 32 rows it stays
-        // with the one-step loop.
+        // with the one-step loop.  Under the rule both loops are kept there (one_step_wins), on
+        // 64 rows the one-step loop alone.
         const ResidentGeom one = g;
         if (params->poisson_loop == EHD_LOOP_AUTO && fixed_ty == 0 && s->rg.cluster.size == 0 &&
-            !(one.TY > 32 && params->poisson_fixed_iter == 1) && fits(2) && g.TY == one.TY &&
-            g.nty == one.nty)
+            !(one.TY > 32 && params->poisson_fixed_iter == 1) &&
+            !(one.TY > 56 && params->poisson_fixed_iter == 0) && fits(2) && g.TY == one.TY &&
+            g.nty == one.nty) {
+          s->other.rg = s->rg;
+          s->other.rthreads = s->rthreads;
+          s->other.rsmem = s->rsmem;
+          s->two_forms = one.TY > 32 && params->poisson_fixed_iter == 0;
           take();
+        }
       }
     }
     cudaGetLastError();
@@ -707,13 +770,14 @@ int sim_create(const ehd_params* params, void* workspace, size_t workspace_bytes
     ehd_destroy(s);
     return EHD_ERR_CUDA;
   }
-  if (cudaMallocHost(&s->h_ctl, sizeof(Ctl)) != cudaSuccess ||
+  if (cudaMallocHost(&s->h_ctl, 2 * sizeof(Ctl)) != cudaSuccess ||
       cudaMallocHost(&s->h_stats, sizeof(DevStats)) != cudaSuccess ||
       cudaMallocHost(&s->h_stage, sizeof(float) * NIO * (size_t)N) != cudaSuccess) {
     cudaGetLastError();
     ehd_destroy(s);
     return EHD_ERR_NOMEM;
   }
+  std::memset(s->h_ctl, 0, 2 * sizeof(Ctl));
   // zero everything once: populations, control, tickets
   if (cudaMemsetAsync(s->ws, 0, L.total, s->stream) != cudaSuccess ||
       cudaStreamSynchronize(s->stream) != cudaSuccess) {
@@ -756,7 +820,7 @@ int ehd_profile_read(ehd_sim* s, ehd_kernel_times* out) {
 void ehd_destroy(ehd_sim* s) {
   if (!s) return;
   cudaStreamSynchronize(s->stream);
-  destroy_graphs(s);
+  forget_graphs(s);
   for (cudaEvent_t e : s->ev) cudaEventDestroy(e);
   for (cudaEvent_t e : s->pev)
     if (e) cudaEventDestroy(e);
@@ -832,8 +896,7 @@ int ehd_set_fields(ehd_sim* s, const void* phi, const void* q, const void* ux, c
     choose_scales(s, m[0], m[1] > m[2] ? m[1] : m[2]);
     // the step graphs hold the coefficients: they stay where the scales, powers of two, do
     if (std::memcmp(old, s->kp.psc, sizeof(old)) != 0) {
-      destroy_graphs(s);
-      s->graphs_tried = false;
+      forget_graphs(s);
     }
   }
   s->n = s->P.start_step;
@@ -845,7 +908,10 @@ int ehd_set_fields(ehd_sim* s, const void* phi, const void* q, const void* ux, c
   EHD_CUDA(launch_step_set(s->kp, s->b, s->cur, s->n, 1, s->stream));
   EHD_LAUNCH(s, 0, launch_init(s->kp, s->b, s->cur, p != nullptr, s->stream));
   s->last_k = 1;
-  return ehd_solve_potential(s, 0.0, 0, nullptr, nullptr);
+  first_form(s);
+  st = ehd_solve_potential(s, 0.0, 0, nullptr, nullptr);
+  first_form(s);  // a copy of the old state's count that was still queued has arrived by now
+  return st;
 }
 
 static int fill_stats(ehd_sim* s, ehd_stats* out) {
@@ -909,6 +975,7 @@ int ehd_step(ehd_sim* s, int nsteps, ehd_stats* out) {
       s->n += ehd_sim::MULTI_STEPS;
       s->history_valid = true;
       k += ehd_sim::MULTI_STEPS - 1;
+      if (follow_count(s, ehd_sim::MULTI_STEPS) != EHD_OK) return EHD_ERR_CUDA;
       continue;
     }
     if (use_graphs && s->profiling) {
@@ -927,6 +994,7 @@ int ehd_step(ehd_sim* s, int nsteps, ehd_stats* out) {
       // the whole step, potential loop included, without returning to the host
       EHD_CUDA(cudaGraphLaunch(s->exec[s->cur], s->stream));
       s->graph_steps += 1;
+      if (follow_count(s, 1) != EHD_OK) return EHD_ERR_CUDA;
     } else {
       {
         NvtxRange r("moments");
@@ -1121,8 +1189,7 @@ int ehd_load_state(ehd_sim* s, const void* buf, size_t bytes) {
       s->kp.psc[f] = hd.psc[f];
       s->kp.ipsc[f] = 1.0f / hd.psc[f];
     }
-    destroy_graphs(s);
-    s->graphs_tried = false;
+    forget_graphs(s);
   }
   const Pops pc = pops_copy(s->kp, s->b, 0);
   if (s->kp.half) {
@@ -1150,6 +1217,7 @@ int ehd_load_state(ehd_sim* s, const void* buf, size_t bytes) {
   s->last_k = hd.last_k;
   EHD_CUDA(launch_step_set(s->kp, s->b, 0, s->n, s->history_valid ? 0 : 1, s->stream));
   EHD_CUDA(cudaStreamSynchronize(s->stream));
+  first_form(s);
   return EHD_OK;
 }
 

@@ -19,7 +19,27 @@ struct NvtxRange {
   NvtxRange& operator=(const NvtxRange&) = delete;
 };
 
-struct ehd_sim {
+// One form of the potential loop on chip and the step graphs built on it.
+struct LoopForm {
+  ehd::ResidentGeom rg{};
+  int rthreads = 0;
+  size_t rsmem = 0;
+  // one step graph per population copy (moments -> while{potential} -> coupled)
+  bool graphs_tried = false;
+  bool graphs_ok = false;
+  cudaGraph_t graph[2] = {nullptr, nullptr};
+  cudaGraphExec_t exec[2] = {nullptr, nullptr};
+  // several consecutive steps in one graph (from copy 0 and from copy 1): runs of that many
+  // steps pay one graph launch instead of one per step
+  cudaGraphExec_t mexec[2] = {nullptr, nullptr};
+  bool mgraphs_ok = false;
+  // the same step graphs with event-record nodes around the three parts, for profiling
+  bool pgraphs_tried = false;
+  bool pgraphs_ok = false;
+  cudaGraphExec_t pexec[2] = {nullptr, nullptr};
+};
+
+struct ehd_sim : LoopForm {
   using KParams = ehd::KParams;
   using Buffers = ehd::Buffers;
   using Ctl = ehd::Ctl;
@@ -36,7 +56,7 @@ struct ehd_sim {
   int64_t n = 0;            // step counter
   bool history_valid = false;
   int last_k = 1;           // sub-iterations of the last potential solve
-  Ctl* h_ctl = nullptr;     // pinned mirror of the loop control
+  Ctl* h_ctl = nullptr;     // pinned mirror of the loop control; [1]: of its count, unsynchronised
   DevStats* h_stats = nullptr;
   float* h_stage = nullptr; // pinned staging for host field I/O, NIO * N floats
   int64_t launches = 0;     // kernel launches queued since the statistics were cleared
@@ -51,28 +71,17 @@ struct ehd_sim {
   size_t ev_used = 0;              // pairs recorded and not yet accumulated
   double prof_ms[4] = {0, 0, 0, 0};
   int64_t prof_n[4] = {0, 0, 0, 0};
-  // one step graph per population copy (moments -> while{potential} -> coupled)
-  bool graphs_tried = false;
-  bool graphs_ok = false;
   bool no_graphs = false;     // steps queued kernel by kernel from the host (ehd_use_graphs)
-  cudaGraph_t graph[2] = {nullptr, nullptr};
-  cudaGraphExec_t exec[2] = {nullptr, nullptr};
-  // MULTI_STEPS consecutive steps in one graph (from copy 0 and from copy 1): runs of that
-  // many steps pay one graph launch instead of one per step
-  static constexpr int MULTI_STEPS = 8;
+  static constexpr int MULTI_STEPS = 8;  // of one multi-step graph
   static_assert(MULTI_STEPS % 2 == 0, "a run must leave the copy index unchanged");
-  cudaGraphExec_t mexec[2] = {nullptr, nullptr};
-  bool mgraphs_ok = false;
-  // the same step graphs with event-record nodes around the three parts, for profiling
-  bool pgraphs_tried = false;
-  bool pgraphs_ok = false;
-  cudaGraphExec_t pexec[2] = {nullptr, nullptr};
   cudaEvent_t pev[4] = {nullptr, nullptr, nullptr, nullptr};
-  // resident (on-chip) potential loop, when the lattice fits
-  bool resident_ok = false;
-  ResidentGeom rg{};
-  int rthreads = 0;
-  size_t rsmem = 0;
+  bool resident_ok = false;   // the potential loop runs on chip, in this object's LoopForm
+  // The library's own choice under the stopping rule on tall tiles: the one- and the two-step
+  // loop, of which one is this object's LoopForm and the other waits here (api.cu follow_count).
+  bool two_forms = false;
+  LoopForm other;
+  int form_steps = 0;         // steps since the device's sub-iteration count was last asked for
+  bool want_one = false;      // what that count asked for
 };
 
 

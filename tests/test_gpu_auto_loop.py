@@ -1,0 +1,97 @@
+"""The library's own choice of loop under the stopping rule on tall tiles: steps whose solves settle
+at one sub-iteration (on tiles of 56 rows also at three) move to the one-step loop, the others
+keep the two-step loop, new fields start with it again; the states are those of the two-step
+loop bit for bit (no tolerance).  The count is set by equal smallest and largest counts, which
+the rule's kernels honour whatever the change of the potential."""
+import numpy as np
+import pytest
+
+from paper_2407_01654_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gpu():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2407_01654_gb300 import build
+    build.build()
+    from paper_2407_01654_gb300 import ehd
+    return ehd
+
+
+def setup(nx, ny, k, **over):
+    p = wl.make_params(nx=nx, ny=ny, walls_y=1, eps_l=4.0, sigma_l=0.05, sigma_v=0.01, varphi_top=0.3,
+                       poisson_tol=1e-12, poisson_min_iter=k, poisson_max_iter=k)
+    p.update(over)
+    y, x = np.meshgrid(np.arange(ny), np.arange(nx), indexing="ij")
+    phi = wl.tanh_profile(0.3 * min(nx, ny) - np.hypot(x - nx / 2.1, y - ny / 2.3), 4.0)
+    return p, (phi, 0 * phi, 0 * phi, 0 * phi)
+
+
+# lattice, storage, count, the loop it settles on (2: one step, 3: two steps an exchange)
+CASES = [(300, 300, 0, 1, 2), (300, 300, 1, 1, 2), (300, 300, 0, 2, 3), (300, 300, 0, 3, 3),
+         (256, 256, 0, 1, 3), (512, 1024, 0, 1, 2), (512, 1024, 0, 3, 2), (512, 1024, 0, 5, 3)]
+
+
+@pytest.mark.parametrize("nx,ny,precision,k,settled", CASES)
+def test_settled_counts_choose_the_loop(gpu, nx, ny, precision, k, settled):
+    p, f = setup(nx, ny, k, precision=precision)
+    ends = []
+    for over in (dict(), dict(poisson_loop=3)):
+        s = gpu.Sim({**p, **over})
+        s.set_fields(*f)
+        assert s.loop_kind() == 3
+        for n in (3, 600, 700, 257):  # calls that end between two looks at the count, and odd ones
+            st = s.step(n)
+            assert st["poisson_iters_min"] == st["poisson_iters_max"] == k and st["steps"] == n
+        assert s.loop_kind() == (3 if over else settled)
+        ends.append(s.read_fields())
+        blob = s.save_state()
+        if not over:
+            for again in (lambda: s.set_fields(*f), lambda: s.load_state(blob)):
+                again()
+                assert s.loop_kind() == 3
+                for n in (1200, 300, 300):  # (the host runs ahead of the device inside a call)
+                    s.step(n)
+                assert s.loop_kind() == settled
+        s.close()
+    for name in ends[0]:
+        assert np.array_equal(ends[0][name], ends[1][name]), name
+
+
+def test_tallest_tiles_keep_the_one_step_loop(gpu):
+    """64 rows: the one-step loop under the rule, the two-step loop at a fixed count."""
+    p, f = setup(576, 1024, 2)
+    for over, kind in ((dict(), 2), (dict(poisson_fixed_iter=2), 3)):
+        s = gpu.Sim({**p, **over})
+        s.set_fields(*f)
+        s.step(600)
+        s.step(300)
+        assert s.loop_kind() == kind
+        s.close()
+
+
+def test_single_steps_and_profiling(gpu):
+    """Steps one at a time follow the count too; steps under profiling run the chosen loop."""
+    p, f = setup(300, 300, 1)
+    s = gpu.Sim(p)
+    s.set_fields(*f)
+    for _ in range(1100):
+        s.step(1)
+    assert s.loop_kind() == 2
+    s.profile(True)
+    s.step(4)
+    assert s.profile_read()["potential"]["launches"] == 4
+    s.profile(False)
+    a = s.read_fields()
+    s.close()
+    s = gpu.Sim(dict(p, poisson_loop=3))
+    s.set_fields(*f)
+    s.step(1104)
+    b = s.read_fields()
+    s.close()
+    for name in a:
+        assert np.array_equal(a[name], b[name]), name
