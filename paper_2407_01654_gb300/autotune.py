@@ -1,20 +1,22 @@
 """Autotuner for the per-simulation launch schedule of the coupled step.
 
-For one lattice shape (nx, ny, walls, storage precision) it times every candidate
+For one lattice shape (nx, ny, walls, storage precision) and potential scheme it times every candidate
 schedule of the potential loop -- the streaming kernel (one launch per sub-iteration in a
 graph WHILE node), the resident on-chip loop and the on-chip loops with two and three
 sub-iterations per exchange, each with every tile height of 64-wide tiles (`tile_rows`;
 0 = the built-in choice of about 2048 nodes per tile) -- on a short run with
 a fixed number of sub-iterations, and returns the fastest as parameter overrides.  All
 candidates compute the same bits at a fixed sub-iteration count (the tests check this), so
-tuning changes speed only.  Results are cached per device and lattice shape in a JSON
-file ($EHD_AUTOTUNE_CACHE, else ~/.cache/paper_2407_01654_gb300/autotune.json).
+tuning changes speed only.  Results are cached per device, lattice shape and potential
+scheme, for the library whose kernels were timed, in a JSON file ($EHD_AUTOTUNE_CACHE, else
+~/.cache/paper_2407_01654_gb300/autotune.json).
 
     from paper_2407_01654_gb300 import autotune
     params.update(autotune.tune(params))
 """
 from __future__ import annotations
 
+import hashlib
 import json
 import os
 import time
@@ -45,8 +47,30 @@ def candidates(params):
 
 
 def shape_key(params, device_name):
+    """What a schedule is tuned for.  The conventional potential scheme has a key of its own:
+    the loops are other kernels, and one of them (three sub-iterations per exchange) does not
+    exist for it."""
     return (f"{device_name}|{params['nx']}x{params['ny']}|walls{params['walls_y']}"
-            f"|prec{params['precision']}")
+            f"|prec{params['precision']}" + ("|conv" if params.get("potential_scheme") else ""))
+
+
+def library_id():
+    """Identifies the kernels that timings belong to: a hash of the library's sources and build
+    flags.  Cached schedules of another library are not used, since they say nothing about
+    this one."""
+    from . import build
+    paths = [os.path.abspath(build.__file__)]
+    for d in (build.CSRC, os.path.join(build.ROOT, "include")):
+        try:
+            paths += [os.path.join(d, n) for n in sorted(os.listdir(d))
+                      if n.endswith((".cu", ".cuh", ".h"))]
+        except OSError:
+            pass  # a library installed without its sources
+    h = hashlib.sha256()
+    for p in paths:
+        with open(p, "rb") as fh:
+            h.update(os.path.basename(p).encode() + b"\0" + fh.read() + b"\0")
+    return h.hexdigest()[:16]
 
 
 def cache_path():
@@ -65,9 +89,15 @@ def load_cache(path):
         return {}
 
 
+def cached(path, key):
+    """The cached entry of this key if this library's kernels were timed for it, else None."""
+    hit = load_cache(path).get(key)
+    return hit if hit and hit.get("library") == library_id() else None
+
+
 def store_cache(path, key, entry):
     d = load_cache(path)
-    d[key] = entry
+    d[key] = dict(entry, library=library_id())
     try:
         os.makedirs(os.path.dirname(path), exist_ok=True)
         tmp = path + ".tmp"
@@ -128,7 +158,7 @@ def tune(params, fields=None, steps=20, fixed_iter=32, use_cache=True, timer=Non
     key = shape_key(params, device_name)
     path = cache_path()
     if use_cache:
-        hit = load_cache(path).get(key)
+        hit = cached(path, key)
         if hit:
             return dict(hit["overrides"])
     if fields is None:
@@ -203,7 +233,7 @@ def tune_batch(requests, steps=64, budget=2 << 30, use_cache=True, timer=None,
     key = f"{device_name}|batch|{','.join(shapes)}"
     path = cache_path()
     if use_cache:
-        hit = load_cache(path).get(key)
+        hit = cached(path, key)
         if hit:
             return dict(hit["overrides"])
     timer = timer or time_batch_candidate
