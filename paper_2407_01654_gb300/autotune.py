@@ -1,14 +1,14 @@
 """Autotuner for the per-simulation launch schedule of the coupled step.
 
-For one lattice shape (nx, ny, walls, storage precision) and potential scheme it times every candidate
-schedule of the potential loop -- the streaming kernel (one launch per sub-iteration in a
+For one lattice shape (nx, ny, walls, storage precision), potential scheme and kind of count
+(the stopping rule's or a fixed one) it times every candidate schedule of the potential loop -- the streaming kernel (one launch per sub-iteration in a
 graph WHILE node), the resident on-chip loop and the on-chip loops with two and three
 sub-iterations per exchange, each with every tile height of 64-wide tiles (`tile_rows`;
 0 = the built-in choice of about 2048 nodes per tile) -- on a short run with
-a fixed number of sub-iterations, and returns the fastest as parameter overrides.  All
+a set number of sub-iterations, and returns the fastest as parameter overrides.  All
 candidates compute the same bits at a fixed sub-iteration count (the tests check this), so
-tuning changes speed only.  Results are cached per device, lattice shape and potential
-scheme, for the library whose kernels were timed, in a JSON file ($EHD_AUTOTUNE_CACHE, else
+tuning changes speed only.  Results are cached per device and shape_key, for the library whose
+kernels were timed, in a JSON file ($EHD_AUTOTUNE_CACHE, else
 ~/.cache/paper_2407_01654_gb300/autotune.json).
 
     from paper_2407_01654_gb300 import autotune
@@ -49,9 +49,10 @@ def candidates(params):
 def shape_key(params, device_name):
     """What a schedule is tuned for.  The conventional potential scheme has a key of its own:
     the loops are other kernels, and one of them (three sub-iterations per exchange) does not
-    exist for it."""
+    exist for it.  So has a fixed count, which runs another kernel than the stopping rule."""
     return (f"{device_name}|{params['nx']}x{params['ny']}|walls{params['walls_y']}"
-            f"|prec{params['precision']}" + ("|conv" if params.get("potential_scheme") else ""))
+            f"|prec{params['precision']}" + ("|conv" if params.get("potential_scheme") else "")
+            + ("|fixed" if params.get("poisson_fixed_iter") else ""))
 
 
 def library_id():
@@ -124,11 +125,16 @@ def pick(timings):
 
 def time_candidate(params, fields, overrides, steps, fixed_iter):
     """Seconds per step of `steps` coupled steps with `fixed_iter` sub-iterations each,
-    after two warm-up steps; None if the library rejects the schedule."""
+    after two warm-up steps; None if the library rejects the schedule.  Parameters under the
+    stopping rule are timed with the rule's kernels: a smallest count equal to the largest, and
+    a tolerance (within FP32's range when squared) that no solve of that length reaches."""
     from . import ehd
     p = dict(params)
     p.update(overrides)
-    p["poisson_fixed_iter"] = fixed_iter
+    if params.get("poisson_fixed_iter"):
+        p["poisson_fixed_iter"] = fixed_iter
+    else:
+        p.update(poisson_min_iter=fixed_iter, poisson_max_iter=fixed_iter, poisson_tol=1e-12)
     try:
         sim = ehd.Sim(p)
     except ehd.EhdError:

@@ -1,5 +1,5 @@
 """Which cached schedules the autotuner uses (no GPU): none tuned for the other potential scheme,
-none timed on another library's kernels."""
+none timed on another library's kernels, none timed at the other kind of count."""
 import json
 
 import pytest
@@ -60,3 +60,51 @@ def test_a_schedule_of_another_library_is_tuned_again(tuner, edit):
     autotune.tune(p, timer=timer, device_name="dev")
     autotune.tune_batch(reqs, timer=rate, device_name="dev")
     assert calls == []  # and kept from then on
+
+
+class FakeSim:
+    """Records the parameters a candidate is timed with."""
+    seen = []
+
+    def __init__(self, params):
+        FakeSim.seen.append(params)
+        self.params = params
+
+    def loop_kind(self):
+        return self.params["poisson_loop"]
+
+    def set_fields(self, *fields):
+        pass
+
+    def step(self, n, stats=True):
+        pass
+
+    def read_stats(self):
+        pass
+
+    def close(self):
+        pass
+
+
+@pytest.mark.parametrize("count", [0, 5])
+def test_candidates_run_the_kernels_that_the_parameters_run(monkeypatch, tuner, count):
+    """Under the rule the candidates are timed under the rule (its smallest and largest count
+    set), at a fixed count at a fixed one; the two have cached schedules of their own."""
+    from paper_2407_01654_gb300 import ehd
+    path, calls, timer = tuner
+    monkeypatch.setattr(ehd, "Sim", FakeSim)
+    FakeSim.seen = []
+    p = wl.make_params(nx=64, ny=64, poisson_fixed_iter=count)
+    ov = {"poisson_loop": 2, "tile_rows": 32}
+    assert autotune.time_candidate(p, autotune._default_fields(p), ov, 4, 32) >= 0.0
+    q, = FakeSim.seen
+    assert q["poisson_loop"] == 2 and q["tile_rows"] == 32
+    if count:
+        assert q["poisson_fixed_iter"] == 32
+    else:
+        assert q["poisson_fixed_iter"] == 0
+        assert q["poisson_min_iter"] == q["poisson_max_iter"] == 32 and 0 < q["poisson_tol"] < 1e-9
+    autotune.tune(p, timer=timer, device_name="dev")
+    calls.clear()
+    autotune.tune(dict(p, poisson_fixed_iter=0 if count else 5), timer=timer, device_name="dev")
+    assert calls == autotune.candidates(p)
