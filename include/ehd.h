@@ -226,6 +226,13 @@ int ehd_use_graphs(ehd_sim* sim, int enable);
  * it can change between two calls of ehd_step. */
 int ehd_loop_kind(const ehd_sim* sim);
 
+/* Diagnostics: the shape of that loop.  out[0]: ehd_loop_kind; out[1]: CTAs of the
+ * thread-block cluster that runs the whole loop (0: tiles, or streaming); out[2]: lattice rows
+ * of each of them, or of a tile (streaming: 0); out[3]: most nodes such a CTA of the cluster
+ * holds (else 0); out[4]: most sub-iterations of one launch when streaming (on chip: 0, all).
+ * Errors: EHD_ERR_INVALID_ARG (null pointer). */
+int ehd_diag_loop_shape(const ehd_sim* sim, int out[5]);
+
 /* Statistics accumulated since they were last cleared (by ehd_step with stats, or by this
  * call); synchronises the stream and clears them.  Returns the status those steps would
  * have returned. */

@@ -1046,6 +1046,17 @@ int ehd_loop_kind(const ehd_sim* s) {
                           : (s->rg.depth == 2 ? EHD_LOOP_RESIDENT2 : EHD_LOOP_RESIDENT);
 }
 
+int ehd_diag_loop_shape(const ehd_sim* s, int out[5]) {
+  if (!s || !out) return EHD_ERR_INVALID_ARG;
+  const ClusterGeom& c = s->rg.cluster;
+  out[0] = ehd_loop_kind(s);
+  out[1] = s->resident_ok ? c.size : 0;
+  out[2] = !s->resident_ok ? 0 : (c.size > 0 ? c.rows : s->rg.TY);
+  out[3] = s->resident_ok && c.size > 0 ? c.cap : 0;
+  out[4] = s->resident_ok ? 0 : (multi_ok(s->kp) ? multi_depth() : 1);
+  return EHD_OK;
+}
+
 int ehd_read_stats(ehd_sim* s, ehd_stats* out) {
   if (!s || !out) return EHD_ERR_INVALID_ARG;
   if (!s->stats_live) {

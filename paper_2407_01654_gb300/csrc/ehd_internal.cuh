@@ -581,6 +581,7 @@ bool multi_ok(const KParams& kp);
 bool multi_defers(const KParams& kp);
 cudaError_t multi_prepare(const KParams& kp);
 int multi_launches(int fixed);  // launches of a fixed count
+int multi_depth();              // most sub-iterations of a launch
 // fixed: the solve's fixed count, or 0 under the rule.
 cudaError_t launch_poisson_multi(const KParams& kp, const Buffers& b, int fixed, cudaStream_t st);
 cudaError_t add_poisson_multi_node(cudaGraph_t g, const cudaGraphNode_t* deps, size_t nd,

@@ -477,6 +477,7 @@ cudaError_t multi_prepare(const KParams& kp) {
                               (int)Multi<MULTI_D>::SMEM);
 }
 int multi_launches(int fixed) { return (fixed + MULTI_D - 1) / MULTI_D; }
+int multi_depth() { return MULTI_D; }
 
 cudaError_t launch_poisson_multi(const KParams& kp, const Buffers& b, int fixed, cudaStream_t st) {
   KParams k = kp;

@@ -121,6 +121,7 @@ SIGNATURES = {
     "ehd_step": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.POINTER(Stats)]),
     "ehd_read_stats": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(Stats)]),
     "ehd_loop_kind": (ctypes.c_int, [ctypes.c_void_p]),
+    "ehd_diag_loop_shape": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ctypes.c_int)]),
     "ehd_solve_potential": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_double, ctypes.c_int,
                                            ctypes.POINTER(ctypes.c_int),
                                            ctypes.POINTER(ctypes.c_double)]),
@@ -349,8 +350,17 @@ class Sim:
 
     def loop_kind(self):
         """1 streaming loop, 2 on-chip loop, 3 / 4 on-chip loop with two / three
-        sub-iterations per exchange."""
+        sub-iterations per exchange (loop_shape tells the one-cluster form of 2 from its
+        tiles)."""
         return int(lib().ehd_loop_kind(self._h))
+
+    def loop_shape(self):
+        """The shape of that loop: kind as loop_kind; cluster_ctas, rows and capacity of the
+        one-cluster loop (cluster_ctas 0: rows are those of a tile, 0 when streaming);
+        launch_iters, the most sub-iterations of one streaming launch (0 on chip)."""
+        out = (ctypes.c_int * 5)()
+        _check(lib().ehd_diag_loop_shape(self._h, out), "ehd_diag_loop_shape")
+        return dict(zip(("kind", "cluster_ctas", "rows", "capacity", "launch_iters"), out))
 
     def uses_resident_loop(self):
         """True when the potential loop runs on chip (one cooperative launch per solve)."""
