@@ -309,6 +309,7 @@ struct Ctl {
                             // per-CTA partials, reduced by the coupled pass
   int redo;                 // streaming, several sub-iterations a launch: > 0: the rule stopped
                             // the loop inside the last launch; the next one repeats that many
+                            // (one-cluster loop: > 0: a CTA of this solve gave up waiting)
   int plaunch;              // and its launches in the current solve
   unsigned oob;             // checked build: out-of-range indices met (see EHD_IDX)
 };

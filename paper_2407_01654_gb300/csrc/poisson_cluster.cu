@@ -6,8 +6,8 @@
 // tile's perimeter to L2 and its import by the neighbours: about 3.5 us whatever the size.
 // Here every exchange stays in the cluster: post-collision populations are pushed to the
 // node they stream to, in the own CTA's shared memory or in a neighbour's (distributed
-// shared memory), and a sub-iteration ends in one hardware cluster barrier (a CTA barrier
-// when the lattice needs only one CTA).
+// shared memory), and a sub-iteration ends in a CTA barrier and, where there are neighbours,
+// with the arrival of their rows, counted on an mbarrier.
 //
 // Decomposition: CTA r of C owns the rows [r rows, (r + 1) rows) of the lattice, so x stays
 // inside a CTA and only a CTA's first and last row push to another one.  A thread owns NPT
@@ -116,6 +116,22 @@ __device__ __forceinline__ void cluster_arrive() {
 }
 __device__ __forceinline__ void cluster_wait() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// __syncthreads_or for a place that not every warp of the CTA comes through: the hardware joins a
+// barrier's arrivals wherever in the code they come from.
+__device__ __forceinline__ bool cta_or(bool v) {
+  unsigned r;
+  __syncwarp();
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %1, 0;\n\t"
+      "bar.red.or.pred q, 0, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"((unsigned)v)
+      : "memory");
+  return r != 0u;
 }
 
 // Warp sums of x and y in five shuffles: after the first, the low half of the warp carries x
@@ -330,6 +346,8 @@ __global__ void __launch_bounds__(ClusterShape<CAP, NPT>::LAUNCH, 1)
   // v, in the order of the one-step tiled loop: per thread of a 64 x TY tile the nodes of one
   // column TY / 4 rows apart, then lanes, warps and tiles.  Every node leaves its change and
   // its old potential in scratch; the cluster's warps share out the tiles' warps.
+  // A CTA that had given up took part in the first meeting on its way out and is gone: nothing
+  // may be sent to it any more.
   auto tiled_sums = [&](int st, float& sa, float& sb, const float2 (&v)[NP]) {
     float2 d[NP], vn;
 #pragma unroll
@@ -376,6 +394,7 @@ __global__ void __launch_bounds__(ClusterShape<CAP, NPT>::LAUNCH, 1)
     sa = lane < 16 ? part : other;
     sb = lane < 16 ? other : part;
     meet();  // scratch may be written again
+    if (C > 1 && __ldcg(&ctl->redo) != 0) fail = true;
   };
   // The keeper adds up the CTA's sums of sub-iteration st (after the CTA barrier that followed
   // them) and sends them to every CTA.
@@ -552,6 +571,12 @@ __global__ void __launch_bounds__(ClusterShape<CAP, NPT>::LAUNCH, 1)
       all_sums(p - 1, sa, sb);
       verdict = decide(p - 1, sa, sb, false);
       if (verdict == UNSURE) {
+        // a wait that ran out may have left another warp with another verdict: it is at the
+        // barriers at the end of the phase, and these are the same two
+        if (cta_or(fail)) {
+          cta_or(fail);
+          return 2;
+        }
         load_state(OLD);
         tiled_sums(p - 1, sa, sb, v1);
         verdict = decide(p - 1, sa, sb, true);
@@ -641,8 +666,13 @@ __global__ void __launch_bounds__(ClusterShape<CAP, NPT>::LAUNCH, 1)
     }
   }
   if (end == 2) {
-    if (tid == 0) atomicOr(&ctl->bar_error, 1);
-    if (C > 1) {  // every CTA's waits run out: none leaves before the others have stopped too
+    if (tid == 0) {
+      atomicOr(&ctl->bar_error, 1);
+      atomicOr(&ctl->redo, 1);  // tells a CTA that meets this one in tiled_sums
+    }
+    // every CTA's waits run out, or it meets this one: none leaves before the others have
+    // stopped pushing to it
+    if (C > 1) {
       cluster_arrive();
       cluster_wait();
     }
