@@ -57,8 +57,9 @@ enum { EHD_FP32 = 0, EHD_FP16DEV = 1 };
  * with the populations held on chip (only for lattices that fit, about 600k nodes on a
  * GB300; with the library's own tiles, lattices up to about 46k nodes run on one
  * thread-block cluster); AUTO picks RESIDENT where it fits, RESIDENT2 where that fits the
- * same tiles beyond one cluster, and under the stopping rule on tiles above 32 rows the one of
- * the two that the counts of the steps so far ask for. */
+ * same tiles beyond one cluster (under the stopping rule beyond about 39k nodes).  Under the
+ * rule it picks between the tiled one-step loop and RESIDENT2 on tiles above 32 rows, or the
+ * largest clusters, by the counts of the steps so far. */
 enum {
   EHD_LOOP_AUTO = 0,
   EHD_LOOP_STREAM = 1,

@@ -416,10 +416,11 @@ void ensure_graphs(ehd_sim* s) {
   s->mgraphs_ok = mok;
 }
 
-// Under the rule a cycle of the two-step loop makes two sub-iterations whether the second is
-// wanted or not, which on tall tiles costs more than the exchange it saves where the solve
-// takes one, and on the tallest where it takes three.  A step with the one- and the two-step
-// loop in us, by rows of a tile (lattice):
+// Whether the tiled one-step loop is the faster one of a simulation's two forms at k
+// sub-iterations a solve, under the rule; a step in us, the one-step loop first.
+// Against two sub-iterations per exchange: a cycle makes two whether the second is wanted or
+// not, which on tall tiles costs more than the exchange it saves where the solve takes one,
+// and on the tallest where it takes three.  By rows of a tile (lattice):
 //   K = 1   32 (512 x 512) 29.8, 29.6;  40 (512 x 700) 36.2, 37.5;  48 (512 x 800) 40.0, 41.5;
 //           56 (512 x 1024) 47.4, 50.1
 //   K = 3   40 44.5, 43.0;  48 47.9, 47.4;  56 55.8, 57.5
@@ -427,14 +428,23 @@ void ensure_graphs(ehd_sim* s) {
 // (On 64 rows, 576 x 1024, the rule's two-step loop is the slower one at every count, 62.4
 // against 54.2 at K = 1, 80.7 against 72.0 at K = 5, 149.5 against 142.6 at K = 21: it is not
 // taken there at all.)
-bool one_step_wins(int rows, int k) { return rows > 32 && (k == 1 || (k == 3 && rows >= 56)); }
+// Against the largest cluster: 16 SMs read and write the state of up to 46 000 nodes, which a
+// short solve does not win back.  At 180 x 256
+//   K = 1, 2, 3, 5   20.8, 21.8;  24.6, 25.0;  28.2, 28.2;  35.7, 33.9
+bool one_step_wins(const ehd_sim* s, int k) {
+  if (s->rg.cluster.size > 0 || s->other.rg.cluster.size > 0) return k == 1 || k == 2;
+  return s->rg.TY > 32 && (k == 1 || (k == 3 && s->rg.TY >= 56));
+}
 
-void swap_forms(ehd_sim* s) { std::swap(static_cast<LoopForm&>(*s), s->other); }
+void swap_forms(ehd_sim* s) {
+  std::swap(static_cast<LoopForm&>(*s), s->other);
+  s->one_step = !s->one_step;
+}
 
-// The two-step loop, before the count of the new state's solves is known.
+// The other form, for long solves, before the count of the new state's solves is known.
 void first_form(ehd_sim* s) {
   if (!s->two_forms) return;
-  if (s->rg.depth != 2) swap_forms(s);
+  if (s->one_step) swap_forms(s);
   s->form_steps = 0;
   s->want_one = false;
   s->h_ctl[1].iter = 0;
@@ -449,8 +459,8 @@ int follow_count(ehd_sim* s, int steps) {
   if (!s->two_forms || (s->form_steps += steps) < EVERY) return EHD_OK;
   s->form_steps = 0;
   const int k = *static_cast<volatile int*>(&s->h_ctl[1].iter);
-  const bool want_one = one_step_wins(s->rg.TY, k);
-  if (want_one == s->want_one && want_one != (s->rg.depth == 0)) {
+  const bool want_one = one_step_wins(s, k);
+  if (want_one == s->want_one && want_one != s->one_step) {
     swap_forms(s);
     ensure_graphs(s);
     if (!s->graphs_ok) {
@@ -728,16 +738,19 @@ int sim_create(const ehd_params* params, void* workspace, size_t workspace_bytes
       const int depth = loop_depth(params->poisson_loop);
       if (fits(depth)) {
         take();
-        // the library's own choice of tiles: a lattice that fits one cluster's shared
-        // memory runs its loop there (the tiles stay laid out for the diagnostics)
-        ClusterGeom cg;
+        // The library's own choice of tiles.  A lattice that fits one cluster's shared memory
+        // runs its loop there (the tiles stay laid out for the diagnostics), under the rule up
+        // to 2432 nodes a CTA: with more the two-step loop is the faster one at every count
+        // from 2 on (22.6 against 25.0 us a step at K = 2 and 180 x 256, 32.8 against 33.9 at
+        // K = 5; at 187 x 194, 2432 nodes a CTA, 31.5 against 29.3).
+        ClusterGeom cg{};
         if (depth == 0 && fixed_ty == 0)
-          for (int most = 16; most >= 8; most -= 8)
-            if (cluster_geometry(s->kp, &cg, most) && cluster_usable(s->kp, cg)) {
-              s->rg.cluster = cg;
-              break;
-            }
-        // and the other lattices run two sub-iterations per exchange where that fits the same
+          for (int most = 16; most >= 8 && cg.size == 0; most -= 8)
+            if (!cluster_geometry(s->kp, &cg, most) || !cluster_usable(s->kp, cg))
+              cg = ClusterGeom{};
+        const bool rule = params->poisson_fixed_iter == 0;
+        const bool large = cg.size > 0 && cg.cap > 2432 && rule;
+        // The other lattices run two sub-iterations per exchange where that fits the same
         // tiles, whose sums and so decisions are the one-step loop's bit for bit: 3.77 -> 2.27 us
         // per sub-iteration at 256 x 256 under the rule; a fixed count, which has an ending of
         // its own, takes 16.2 us a solve at K = 3 and 512 x 1024 against 21.8.
@@ -745,15 +758,17 @@ int sim_create(const ehd_params* params, void* workspace, size_t workspace_bytes
         // with the one-step loop.  Under the rule both loops are kept there (one_step_wins), on
         // 64 rows the one-step loop alone.
         const ResidentGeom one = g;
-        if (params->poisson_loop == EHD_LOOP_AUTO && fixed_ty == 0 && s->rg.cluster.size == 0 &&
-            !(one.TY > 32 && params->poisson_fixed_iter == 1) &&
-            !(one.TY > 56 && params->poisson_fixed_iter == 0) && fits(2) && g.TY == one.TY &&
-            g.nty == one.nty) {
-          s->other.rg = s->rg;
-          s->other.rthreads = s->rthreads;
-          s->other.rsmem = s->rsmem;
-          s->two_forms = one.TY > 32 && params->poisson_fixed_iter == 0;
+        s->other.rg = s->rg;
+        s->other.rthreads = s->rthreads;
+        s->other.rsmem = s->rsmem;
+        if (params->poisson_loop == EHD_LOOP_AUTO && fixed_ty == 0 && (cg.size == 0 || large) &&
+            !(one.TY > 32 && params->poisson_fixed_iter == 1) && !(one.TY > 56 && rule) &&
+            fits(2) && g.TY == one.TY && g.nty == one.nty) {
           take();
+          s->two_forms = one.TY > 32 && rule;
+        } else {
+          s->rg.cluster = cg;
+          s->two_forms = large;
         }
       }
     }

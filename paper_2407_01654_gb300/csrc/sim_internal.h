@@ -76,9 +76,11 @@ struct ehd_sim : LoopForm {
   static_assert(MULTI_STEPS % 2 == 0, "a run must leave the copy index unchanged");
   cudaEvent_t pev[4] = {nullptr, nullptr, nullptr, nullptr};
   bool resident_ok = false;   // the potential loop runs on chip, in this object's LoopForm
-  // The library's own choice under the stopping rule on tall tiles: the one- and the two-step
-  // loop, of which one is this object's LoopForm and the other waits here (api.cu follow_count).
+  // The library's own choice under the stopping rule, where it goes by the count: the tiled
+  // one-step loop and the two-step loop on tall tiles or the largest cluster, of which one is
+  // this object's LoopForm and the other waits here (api.cu follow_count).
   bool two_forms = false;
+  bool one_step = false;      // the tiled one-step loop is this object's
   LoopForm other;
   int form_steps = 0;         // steps since the device's sub-iteration count was last asked for
   bool want_one = false;      // what that count asked for

@@ -1,7 +1,8 @@
-"""The library's own choice of loop under the stopping rule on tall tiles: steps whose solves settle
+"""The library's own choice of loop under the stopping rule: on tall tiles steps whose solves settle
 at one sub-iteration (on tiles of 56 rows also at three) move to the one-step loop, the others
-keep the two-step loop, new fields start with it again; the states are those of the two-step
-loop bit for bit (no tolerance).  The count is set by equal smallest and largest counts, which
+keep the two-step loop; with the largest cluster, where the two-step loop does not fit, one and
+two sub-iterations move.  New fields start with the other form again; the states are those of
+one loop bit for bit (no tolerance).  The count is set by equal smallest and largest counts, which
 the rule's kernels honour whatever the change of the potential."""
 import numpy as np
 import pytest
@@ -31,32 +32,41 @@ def setup(nx, ny, k, **over):
     return p, (phi, 0 * phi, 0 * phi, 0 * phi)
 
 
-# lattice, storage, count, the loop it settles on (2: one step, 3: two steps an exchange)
-CASES = [(300, 300, 0, 1, 2), (300, 300, 1, 1, 2), (300, 300, 0, 2, 3), (300, 300, 0, 3, 3),
+# lattice, storage, count, the loop it settles on (2: one step, 3: two steps an exchange, 0: cluster)
+CASES = [(200, 200, 0, 1, 2), (200, 200, 0, 2, 3), (193, 224, 0, 1, 2), (193, 224, 1, 2, 2),
+         (193, 224, 0, 3, 0),
+         (300, 300, 0, 1, 2), (300, 300, 1, 1, 2), (300, 300, 0, 2, 3), (300, 300, 0, 3, 3),
          (256, 256, 0, 1, 3), (512, 1024, 0, 1, 2), (512, 1024, 0, 3, 2), (512, 1024, 0, 5, 3)]
+
+
+def loop_of(s):
+    d = s.loop_shape()
+    return 0 if d["cluster_ctas"] else d["kind"]
 
 
 @pytest.mark.parametrize("nx,ny,precision,k,settled", CASES)
 def test_settled_counts_choose_the_loop(gpu, nx, ny, precision, k, settled):
     p, f = setup(nx, ny, k, precision=precision)
     ends = []
-    for over in (dict(), dict(poisson_loop=3)):
+    first = 0 if nx == 193 else 3
+    one_loop = dict(poisson_loop=3) if first else dict(poisson_loop=2, tile_rows=32)
+    for over in (dict(), one_loop):
         s = gpu.Sim({**p, **over})
         s.set_fields(*f)
-        assert s.loop_kind() == 3
+        assert loop_of(s) == (over.get("poisson_loop") or first)
         for n in (3, 600, 700, 257):  # calls that end between two looks at the count, and odd ones
             st = s.step(n)
             assert st["poisson_iters_min"] == st["poisson_iters_max"] == k and st["steps"] == n
-        assert s.loop_kind() == (3 if over else settled)
+        assert loop_of(s) == (over.get("poisson_loop") or settled)
         ends.append(s.read_fields())
         blob = s.save_state()
         if not over:
             for again in (lambda: s.set_fields(*f), lambda: s.load_state(blob)):
                 again()
-                assert s.loop_kind() == 3
+                assert loop_of(s) == first
                 for n in (1200, 300, 300):  # (the host runs ahead of the device inside a call)
                     s.step(n)
-                assert s.loop_kind() == settled
+                assert loop_of(s) == settled
         s.close()
     for name in ends[0]:
         assert np.array_equal(ends[0][name], ends[1][name]), name

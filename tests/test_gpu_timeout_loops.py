@@ -40,7 +40,7 @@ CASES = {
     "three-step-rule": (96, dict(poisson_loop=4, tile_rows=48), dict(kind=4, rows=48)),
     "cluster-rule": (96, dict(), dict(kind=2, cluster_ctas=16, capacity=768)),
     "cluster-fixed": (96, dict(poisson_fixed_iter=5), dict(kind=2, cluster_ctas=16, capacity=768)),
-    "cluster-two-copies-rule": (200, dict(), dict(kind=2, cluster_ctas=16, capacity=2880)),
+    "cluster-two-copies-rule": (187, dict(), dict(kind=2, cluster_ctas=16, capacity=2432)),
     "cluster-two-copies-fixed": (200, dict(poisson_fixed_iter=5),
                                  dict(kind=2, cluster_ctas=16, capacity=2880)),
     "one-cta": (16, dict(), dict(kind=2, cluster_ctas=1)),
