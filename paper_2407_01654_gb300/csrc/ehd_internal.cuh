@@ -311,6 +311,7 @@ struct Ctl {
                             // the loop inside the last launch; the next one repeats that many
                             // (one-cluster loop: > 0: a CTA of this solve gave up waiting)
   int plaunch;              // and its launches in the current solve
+  int guess;                // and the sub-iterations of the last solve (0: not known)
   unsigned oob;             // checked build: out-of-range indices met (see EHD_IDX)
 };
 

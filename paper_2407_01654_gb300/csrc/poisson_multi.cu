@@ -18,7 +18,11 @@
 // block that a thread of it owns; FP32 in a warp, FP64 beyond), so a decision differs only
 // where FP64 sums in another order do.  The last CTA applies the rule to the n sub-iterations in
 // order.  When it stops the loop before the n-th, the state in the other copy of h, from which
-// this launch began, is advanced again by that many: one more launch per solve at most.
+// this launch began, is advanced again by that many: one more launch per solve at most.  So that
+// settled solves need none, a launch aims at the count that the solve before took (multi_steps):
+// with launches of five whatever the count a step took 371, 390, 408, 425 and 325 us at K = 1 ... 5
+// and 1024 x 2048, with these it takes 242, 265, 288, 300 and 325, with one sub-iteration a
+// launch 237, 296, 355, 414 and 473.
 //
 // A fixed count needs no decision, so the order of its sums (a statistic) is free and with it
 // the tile height: two CTAs fit an SM, and tiles as tall as the lattice's whole waves of
@@ -51,14 +55,22 @@ __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
                : "memory");
 }
 
-// Sub-iterations the next launch makes: what is left of a fixed count in equal launches, or
-// under the rule as many as it may.
-__host__ __device__ inline int multi_steps(int d, int fixed, int max_iter, int iter) {
+// Sub-iterations the next launch makes.  A fixed count: what is left of it in equal launches.
+// Under the rule: the same up to the count of the solve before (`guess`, 0: not known), which the
+// next solve mostly takes again, so that the launch that ends it ends where the rule does; past
+// it one, two, four and then all that a launch may make.
+__device__ inline int multi_steps(int d, int fixed, int max_iter, int iter, int guess) {
   const int left = (fixed > 0 ? fixed : max_iter) - iter;
-  if (left <= d) return left;
-  if (fixed <= 0) return d;
-  const int launches = (left + d - 1) / d;
-  return (left + launches - 1) / launches;
+  int aim = left;
+  if (fixed <= 0) {
+    if (guess <= 0) return left < d ? left : d;
+    const int past = iter - guess;
+    aim = past < 0 ? -past : (past + 1 < d ? past + 1 : d);
+    if (aim > left) aim = left;
+  }
+  if (aim <= d) return aim;
+  const int launches = (aim + d - 1) / d;
+  return (aim + launches - 1) / launches;
 }
 
 }  // namespace
@@ -85,7 +97,7 @@ __global__ void __launch_bounds__(MT, 2)
   const int fixed = bad_state ? 0 : __ldg(&ctl->fixed_iter),
             max_iter = bad_state ? 1 : __ldg(&ctl->max_iter);
   const int iter = __ldg(&ctl->iter), redo = __ldg(&ctl->redo);
-  const int n = redo > 0 ? redo : multi_steps(D, fixed, max_iter, iter);
+  const int n = redo > 0 ? redo : multi_steps(D, fixed, max_iter, iter, __ldg(&ctl->guess));
   const int nx = k.nx, ny = k.ny;
   const size_t N = (size_t)k.N;
   const float* __restrict__ src = hbuf + (size_t)parity * NH * N;
@@ -404,6 +416,7 @@ __global__ void __launch_bounds__(MT, 2)
       ctl->rel = rel;
       ctl->converged = conv;
     }
+    if (done) ctl->guess = iter + stop;
     if (done && stop < n) {
       ctl->redo = stop;  // the next launch repeats this one's first sub-iterations
       done = 0;
@@ -460,7 +473,7 @@ const void* multi_kernel(const KParams& kp) {
 
 // Lattices that stream several sub-iterations per launch: those beyond the chip's storage, as
 // long as the partial sums of every sub-iteration of a launch have room (a fixed count's lower
-// tiles, at most three times as many, keep only one sub-iteration's).
+// tiles, little more than twice as many, keep only one sub-iteration's).
 bool multi_ok(const KParams& kp) {
   return !kp.slab && (long long)kp.nx * kp.ny > MULTI_MIN_NODES &&
          (long long)multi_blocks(kp) * MULTI_D <= MAX_PARTIALS;
