@@ -53,7 +53,7 @@ enum { EHD_HOST = 0, EHD_DEVICE = 1 };
 enum { EHD_FP32 = 0, EHD_FP16DEV = 1 };
 /* Implementation of the potential sub-iteration loop (same arithmetic, same results):
  * STREAM runs kernels over populations in device memory, one per sub-iteration (above 600k
- * nodes up to five sub-iterations per kernel); RESIDENT runs the whole loop in one kernel
+ * nodes up to five sub-iterations per kernel, except where the rule settles at one); RESIDENT runs the whole loop in one kernel
  * with the populations held on chip (only for lattices that fit, about 600k nodes on a
  * GB300; with the library's own tiles, lattices up to about 46k nodes run on one
  * thread-block cluster); AUTO picks RESIDENT where it fits, RESIDENT2 where that fits the

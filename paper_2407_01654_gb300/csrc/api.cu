@@ -263,6 +263,9 @@ void prof_end(ehd_sim* s, long j) {
     if (e_ != cudaSuccess) return EHD_ERR_CUDA; \
   } while (0)
 
+// Whether the moments pass may leave its sums to the coupled pass (launch_moments).
+bool tail_free(const ehd_sim* s) { return s->resident_ok || (s->multi && multi_defers(s->kp)); }
+
 // The potential loop of one solve.  The moments kernel has reset the control.  Fixed
 // count: exactly that many launches.  Stopping rule: launches are queued in chunks; a
 // launch after the rule has fired returns at once; the pinned control mirror tells the
@@ -286,7 +289,7 @@ int run_potential_loop(ehd_sim* s, int fixed, int max_iter) {
     s->last_k = s->h_ctl->iter;
     return s->h_ctl->converged ? EHD_OK : EHD_ERR_NOT_CONVERGED;
   }
-  const bool multi = multi_ok(s->kp);
+  const bool multi = s->multi;
   auto launch = [&]() {
     return multi ? launch_poisson_multi(s->kp, s->b, fixed, s->stream)
                  : launch_poisson(s->kp, s->b, s->stream);
@@ -363,7 +366,7 @@ void ensure_prof_graphs(ehd_sim* s) {
     const bool ok =
         build_step_graph(s->kp, s->b, c, P.poisson_tol, P.poisson_min_iter, P.poisson_max_iter,
                          P.poisson_fixed_iter, s->resident_ok ? &s->rg : nullptr, s->rthreads,
-                         s->rsmem, &g, s->pev) == cudaSuccess &&
+                         s->rsmem, s->multi, &g, s->pev) == cudaSuccess &&
         cudaGraphInstantiate(&s->pexec[c], g, 0) == cudaSuccess;
     if (g) cudaGraphDestroy(g);
     if (!ok) {
@@ -387,7 +390,7 @@ void ensure_graphs(ehd_sim* s) {
   for (int c = 0; c < 2; ++c) {
     if (build_step_graph(s->kp, s->b, c, P.poisson_tol, P.poisson_min_iter, P.poisson_max_iter,
                          P.poisson_fixed_iter, s->resident_ok ? &s->rg : nullptr, s->rthreads,
-                         s->rsmem, &s->graph[c]) != cudaSuccess ||
+                         s->rsmem, s->multi, &s->graph[c]) != cudaSuccess ||
         cudaGraphInstantiate(&s->exec[c], s->graph[c], 0) != cudaSuccess) {
       cudaGetLastError();
       destroy_graphs(s);
@@ -401,8 +404,8 @@ void ensure_graphs(ehd_sim* s) {
     cudaGraph_t g = nullptr;
     mok = build_step_graph(s->kp, s->b, c, P.poisson_tol, P.poisson_min_iter,
                            P.poisson_max_iter, P.poisson_fixed_iter,
-                           s->resident_ok ? &s->rg : nullptr, s->rthreads, s->rsmem, &g,
-                           nullptr, ehd_sim::MULTI_STEPS) == cudaSuccess &&
+                           s->resident_ok ? &s->rg : nullptr, s->rthreads, s->rsmem,
+                           s->multi, &g, nullptr, ehd_sim::MULTI_STEPS) == cudaSuccess &&
           cudaGraphInstantiate(&s->mexec[c], g, 0) == cudaSuccess;
     if (g) cudaGraphDestroy(g);
   }
@@ -416,8 +419,8 @@ void ensure_graphs(ehd_sim* s) {
   s->mgraphs_ok = mok;
 }
 
-// Whether the tiled one-step loop is the faster one of a simulation's two forms at k
-// sub-iterations a solve, under the rule; a step in us, the one-step loop first.
+// Whether one sub-iteration at a time is the faster one of a simulation's two forms at k
+// sub-iterations a solve, under the rule; a step in us, this form first.
 // Against two sub-iterations per exchange: a cycle makes two whether the second is wanted or
 // not, which on tall tiles costs more than the exchange it saves where the solve takes one,
 // and on the tallest where it takes three.  By rows of a tile (lattice):
@@ -431,7 +434,10 @@ void ensure_graphs(ehd_sim* s) {
 // Against the largest cluster: 16 SMs read and write the state of up to 46 000 nodes, which a
 // short solve does not win back.  At 180 x 256
 //   K = 1, 2, 3, 5   20.8, 21.8;  24.6, 25.0;  28.2, 28.2;  35.7, 33.9
+// Beyond the chip's storage the one-sub-iteration launch is the better one of its kind: at K = 1
+// 75.3, 78.0 (1000 x 601); 106.7, 112.7 (977 x 811); 237.0, 242.5 (1024 x 2048).
 bool one_step_wins(const ehd_sim* s, int k) {
+  if (!s->resident_ok) return k == 1;
   if (s->rg.cluster.size > 0 || s->other.rg.cluster.size > 0) return k == 1 || k == 2;
   return s->rg.TY > 32 && (k == 1 || (k == 3 && s->rg.TY >= 56));
 }
@@ -780,10 +786,14 @@ int sim_create(const ehd_params* params, void* workspace, size_t workspace_bytes
       return EHD_ERR_INVALID_ARG;  // the lattice does not fit on chip on this device
     }
   }
-  if (!s->resident_ok && multi_ok(s->kp) && multi_prepare(s->kp) != cudaSuccess) {
-    cudaGetLastError();
-    ehd_destroy(s);
-    return EHD_ERR_CUDA;
+  if (!s->resident_ok && multi_ok(s->kp)) {
+    if (multi_prepare(s->kp) != cudaSuccess) {
+      cudaGetLastError();
+      ehd_destroy(s);
+      return EHD_ERR_CUDA;
+    }
+    s->multi = true;  // and under the rule one sub-iteration a launch as the other form
+    s->two_forms = params->poisson_fixed_iter == 0;
   }
   if (cudaMallocHost(&s->h_ctl, 2 * sizeof(Ctl)) != cudaSuccess ||
       cudaMallocHost(&s->h_stats, sizeof(DevStats)) != cudaSuccess ||
@@ -876,7 +886,7 @@ int ehd_solve_potential(ehd_sim* s, double tol, int max_iter, int* iters, double
   const int mx = max_iter > 0 ? max_iter : P.poisson_max_iter;
   const int fixed = (tol > 0 || max_iter > 0) ? 0 : P.poisson_fixed_iter;
   EHD_LAUNCH(s, 0, launch_moments(s->kp, s->b, s->cur, t, P.poisson_min_iter, mx, fixed,
-                                   s->stream, s->resident_ok || multi_defers(s->kp)));
+                                   s->stream, tail_free(s)));
   int st = run_potential_loop(s, fixed, mx);
   if (st == EHD_ERR_CUDA) return st;
   if (!s->resident_ok && fixed > 0) {  // the other loops end with the control read back
@@ -919,7 +929,7 @@ int ehd_set_fields(ehd_sim* s, const void* phi, const void* q, const void* ux, c
   // the populations are written into the current copy; the potential restarts in copy 0
   EHD_CUDA(cudaMemsetAsync(&s->b.ctl->parity, 0, sizeof(int), s->stream));
   EHD_CUDA(cudaMemsetAsync(&s->b.ctl->nonfinite, 0, sizeof(int), s->stream));
-  if (multi_ok(s->kp)) EHD_CUDA(cudaMemsetAsync(&s->b.ctl->guess, 0, sizeof(int), s->stream));
+  if (s->multi) EHD_CUDA(cudaMemsetAsync(&s->b.ctl->guess, 0, sizeof(int), s->stream));
   s->launches += 1;
   EHD_CUDA(launch_step_set(s->kp, s->b, s->cur, s->n, 1, s->stream));
   EHD_LAUNCH(s, 0, launch_init(s->kp, s->b, s->cur, p != nullptr, s->stream));
@@ -948,12 +958,7 @@ static int fill_stats(ehd_sim* s, ehd_stats* out) {
   // host-driven launches are counted as they are queued; a graph step launches moments,
   // the potential loop (one resident kernel, or one kernel per sub-iteration) and coupled
   out->kernel_launches = s->launches + 2LL * s->graph_steps;
-  if (s->resident_ok)
-    out->kernel_launches += s->graph_steps;
-  else if (multi_ok(s->kp))
-    out->kernel_launches += (int64_t)d.plaunches - s->host_iters;
-  else
-    out->kernel_launches += (int64_t)d.iters_total - s->host_iters;
+  out->kernel_launches += s->resident_ok ? s->graph_steps : (int64_t)d.plaunches - s->host_iters;
   int status = EHD_OK;
   if (d.not_converged) status = EHD_ERR_NOT_CONVERGED;
   if (d.nonfinite) status = EHD_ERR_NONFINITE;
@@ -1017,7 +1022,7 @@ int ehd_step(ehd_sim* s, int nsteps, ehd_stats* out) {
         EHD_LAUNCH(s, 0, launch_moments(s->kp, s->b, s->cur, P.poisson_tol,
                                          P.poisson_min_iter, P.poisson_max_iter,
                                          P.poisson_fixed_iter, s->stream,
-                                         s->resident_ok || multi_defers(s->kp)));
+                                         tail_free(s)));
       }
       int st;
       {
@@ -1026,7 +1031,7 @@ int ehd_step(ehd_sim* s, int nsteps, ehd_stats* out) {
       }
       if (st == EHD_ERR_CUDA || st == EHD_ERR_TIMEOUT) return st;
       if (st != EHD_OK) status = st;
-      if (!s->resident_ok) s->host_iters += multi_ok(s->kp) ? s->h_ctl->plaunch : s->h_ctl->iter;
+      if (!s->resident_ok) s->host_iters += s->h_ctl->plaunch;
       NvtxRange r("coupled");
       EHD_LAUNCH(s, 3, launch_coupled(s->kp, s->b, s->cur, s->stream));
     }
@@ -1069,7 +1074,7 @@ int ehd_diag_loop_shape(const ehd_sim* s, int out[5]) {
   out[1] = s->resident_ok ? c.size : 0;
   out[2] = !s->resident_ok ? 0 : (c.size > 0 ? c.rows : s->rg.TY);
   out[3] = s->resident_ok && c.size > 0 ? c.cap : 0;
-  out[4] = s->resident_ok ? 0 : (multi_ok(s->kp) ? multi_depth() : 1);
+  out[4] = s->resident_ok ? 0 : (s->multi ? multi_depth() : 1);
   return EHD_OK;
 }
 

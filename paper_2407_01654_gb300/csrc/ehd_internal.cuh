@@ -310,8 +310,8 @@ struct Ctl {
   int redo;                 // streaming, several sub-iterations a launch: > 0: the rule stopped
                             // the loop inside the last launch; the next one repeats that many
                             // (one-cluster loop: > 0: a CTA of this solve gave up waiting)
-  int plaunch;              // and its launches in the current solve
-  int guess;                // and the sub-iterations of the last solve (0: not known)
+  int plaunch;              // streaming: launches of the current solve
+  int guess;                // several sub-iterations a launch: those of the last solve (0: not known)
   unsigned oob;             // checked build: out-of-range indices met (see EHD_IDX)
 };
 
@@ -335,7 +335,7 @@ struct ResidentGeom {
 struct DevStats {
   int iters_total, iters_min, iters_max, not_converged, nonfinite, steps;
   int barrier_error;
-  int plaunches;            // streaming launches, where a launch makes several sub-iterations
+  int plaunches;            // streaming launches
   double last_rel, sum_phi, sum_q;
 };
 
@@ -639,13 +639,13 @@ cudaError_t add_coupled_node(cudaGraph_t g, const cudaGraphNode_t* deps, size_t 
 // { potential sub-iteration } -> coupled pass.  All arguments live on the device, so the
 // graph is launched unchanged every step.
 // With `rg` non-null the potential loop is the single resident cooperative kernel instead
-// of the WHILE node.
+// of the WHILE node; else with `multi` streaming launches of several sub-iterations.
 // With `ev` (4 events) the graph records ev[0] before the moments pass, ev[1] after it,
 // ev[2] after the potential loop and ev[3] after the coupled pass (per-kernel timing).
 // With nsteps > 1 (and no events) the graph holds that many consecutive steps, the first
 // on population copy `cur`, the copies alternating: one launch runs them all.
 cudaError_t build_step_graph(const KParams& kp, const Buffers& b, int cur, double tol,
                              int min_iter, int max_iter, int fixed_iter, const ResidentGeom* rg,
-                             int rthreads, size_t rsmem, cudaGraph_t* out,
+                             int rthreads, size_t rsmem, bool multi, cudaGraph_t* out,
                              const cudaEvent_t* ev = nullptr, int nsteps = 1);
 }  // namespace ehd

@@ -1423,7 +1423,7 @@ cudaError_t add_poisson_node(cudaGraph_t g, cudaGraphNode_t* out, const KParams&
 
 cudaError_t build_step_graph(const KParams& kp, const Buffers& b, int cur, double tol,
                              int min_iter, int max_iter, int fixed_iter, const ResidentGeom* rg,
-                             int rthreads, size_t rsmem, cudaGraph_t* out,
+                             int rthreads, size_t rsmem, bool multi, cudaGraph_t* out,
                              const cudaEvent_t* ev, int nsteps) {
   if (nsteps < 1 || (ev && nsteps != 1)) return cudaErrorInvalidValue;
   cudaGraph_t g;
@@ -1457,7 +1457,8 @@ cudaError_t build_step_graph(const KParams& kp, const Buffers& b, int cur, doubl
     cudaGraphNode_t mn, wn, pn, cn;
     if ((e = record(0)) != cudaSuccess ||
         (e = add_moments_node(g, have ? &last : nullptr, have ? 1 : 0, &mn, kp, b, c, tol,
-                              min_iter, max_iter, fixed_iter, rg || multi_defers(kp))) != cudaSuccess)
+                              min_iter, max_iter, fixed_iter,
+                              rg || (multi && multi_defers(kp)))) != cudaSuccess)
       return done(e);
     last = mn;
     have = true;
@@ -1468,7 +1469,7 @@ cudaError_t build_step_graph(const KParams& kp, const Buffers& b, int cur, doubl
           cudaSuccess)
         return done(e);
       last = pn;
-    } else if (multi_ok(kp) && fixed_iter > 0 && multi_launches(fixed_iter) <= 8) {
+    } else if (multi && fixed_iter > 0 && multi_launches(fixed_iter) <= 8) {
       // a fixed count's few launches in a row, without a condition between them (after a
       // non-finite field the first one ends the loop and the others return at once)
       for (int l = 0; l < multi_launches(fixed_iter); ++l) {
@@ -1488,7 +1489,7 @@ cudaError_t build_step_graph(const KParams& kp, const Buffers& b, int cur, doubl
       cp.conditional.type = cudaGraphCondTypeWhile;
       cp.conditional.size = 1;
       if ((e = cudaGraphAddNode(&wn, g, &last, nullptr, 1, &cp)) != cudaSuccess ||
-          (e = multi_ok(kp)
+          (e = multi
                    ? add_poisson_multi_node(cp.conditional.phGraph_out[0], nullptr, 0, &pn, kp, b,
                                             fixed_iter, &h)
                    : add_poisson_node(cp.conditional.phGraph_out[0], &pn, kp, b, h)) != cudaSuccess)

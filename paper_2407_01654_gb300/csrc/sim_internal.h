@@ -19,11 +19,12 @@ struct NvtxRange {
   NvtxRange& operator=(const NvtxRange&) = delete;
 };
 
-// One form of the potential loop on chip and the step graphs built on it.
+// One form of the potential loop and the step graphs built on it.
 struct LoopForm {
-  ehd::ResidentGeom rg{};
+  ehd::ResidentGeom rg{};  // on chip
   int rthreads = 0;
   size_t rsmem = 0;
+  bool multi = false;      // streaming: several sub-iterations a launch
   // one step graph per population copy (moments -> while{potential} -> coupled)
   bool graphs_tried = false;
   bool graphs_ok = false;
@@ -61,7 +62,7 @@ struct ehd_sim : LoopForm {
   float* h_stage = nullptr; // pinned staging for host field I/O, NIO * N floats
   int64_t launches = 0;     // kernel launches queued since the statistics were cleared
   int64_t graph_steps = 0;  // steps run as graphs since then
-  int64_t host_iters = 0;   // potential sub-iterations run from the host loop since then
+  int64_t host_iters = 0;   // streaming launches queued from the host loop since then
   bool stats_live = false;  // device statistics are accumulating
   // per-launch event timing
   bool profiling = false;
@@ -76,11 +77,12 @@ struct ehd_sim : LoopForm {
   static_assert(MULTI_STEPS % 2 == 0, "a run must leave the copy index unchanged");
   cudaEvent_t pev[4] = {nullptr, nullptr, nullptr, nullptr};
   bool resident_ok = false;   // the potential loop runs on chip, in this object's LoopForm
-  // The library's own choice under the stopping rule, where it goes by the count: the tiled
-  // one-step loop and the two-step loop on tall tiles or the largest cluster, of which one is
-  // this object's LoopForm and the other waits here (api.cu follow_count).
+  // Where the best loop under the stopping rule goes by the count: one sub-iteration at a time
+  // (tiles, or streaming launches), or the two-step loop on tall tiles, the largest cluster,
+  // streaming launches of several.  One is this object's LoopForm, the other waits here
+  // (api.cu follow_count).
   bool two_forms = false;
-  bool one_step = false;      // the tiled one-step loop is this object's
+  bool one_step = false;      // one sub-iteration at a time is this object's
   LoopForm other;
   int form_steps = 0;         // steps since the device's sub-iteration count was last asked for
   bool want_one = false;      // what that count asked for

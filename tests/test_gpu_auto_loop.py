@@ -1,7 +1,7 @@
 """The library's own choice of loop under the stopping rule: on tall tiles steps whose solves settle
 at one sub-iteration (on tiles of 56 rows also at three) move to the one-step loop, the others
 keep the two-step loop; with the largest cluster, where the two-step loop does not fit, one and
-two sub-iterations move.  New fields start with the other form again; the states are those of
+two sub-iterations move; beyond the chip's storage one sub-iteration moves to launches of one.  New fields start with the other form again; the states are those of
 one loop bit for bit (no tolerance).  The count is set by equal smallest and largest counts, which
 the rule's kernels honour whatever the change of the potential."""
 import numpy as np
@@ -34,13 +34,15 @@ def setup(nx, ny, k, **over):
 
 # lattice, storage, count, the loop it settles on (2: one step, 3: two steps an exchange, 0: cluster)
 CASES = [(200, 200, 0, 1, 2), (200, 200, 0, 2, 3), (193, 224, 0, 1, 2), (193, 224, 1, 2, 2),
-         (193, 224, 0, 3, 0),
+         (193, 224, 0, 3, 0), (1000, 601, 0, 1, "single"), (1000, 601, 1, 2, "several"),
          (300, 300, 0, 1, 2), (300, 300, 1, 1, 2), (300, 300, 0, 2, 3), (300, 300, 0, 3, 3),
          (256, 256, 0, 1, 3), (512, 1024, 0, 1, 2), (512, 1024, 0, 3, 2), (512, 1024, 0, 5, 3)]
 
 
 def loop_of(s):
     d = s.loop_shape()
+    if d["kind"] == 1:
+        return {1: "single", 5: "several"}[d["launch_iters"]]
     return 0 if d["cluster_ctas"] else d["kind"]
 
 
@@ -48,16 +50,20 @@ def loop_of(s):
 def test_settled_counts_choose_the_loop(gpu, nx, ny, precision, k, settled):
     p, f = setup(nx, ny, k, precision=precision)
     ends = []
-    first = 0 if nx == 193 else 3
-    one_loop = dict(poisson_loop=3) if first else dict(poisson_loop=2, tile_rows=32)
+    first = {193: 0, 1000: "several"}.get(nx, 3)
+    one_loop = {193: dict(poisson_loop=2, tile_rows=32), 1000: dict(poisson_loop=1)}.get(
+        nx, dict(poisson_loop=3))
     for over in (dict(), one_loop):
         s = gpu.Sim({**p, **over})
+        if over.get("poisson_loop") == 1:
+            s.use_graphs(False)  # steps from the host keep their launches of several
         s.set_fields(*f)
-        assert loop_of(s) == (over.get("poisson_loop") or first)
+        stays = {1: first}.get(over.get("poisson_loop"), over.get("poisson_loop"))
+        assert loop_of(s) == (stays or first)
         for n in (3, 600, 700, 257):  # calls that end between two looks at the count, and odd ones
             st = s.step(n)
             assert st["poisson_iters_min"] == st["poisson_iters_max"] == k and st["steps"] == n
-        assert loop_of(s) == (over.get("poisson_loop") or settled)
+        assert loop_of(s) == (stays or settled)
         ends.append(s.read_fields())
         blob = s.save_state()
         if not over:
