@@ -1031,7 +1031,7 @@ int ehd_step(ehd_sim* s, int nsteps, ehd_stats* out) {
       }
       if (st == EHD_ERR_CUDA || st == EHD_ERR_TIMEOUT) return st;
       if (st != EHD_OK) status = st;
-      if (!s->resident_ok) s->host_iters += s->h_ctl->plaunch;
+      if (!s->resident_ok) s->host_iters += s->multi ? s->h_ctl->plaunch : s->h_ctl->iter;
       NvtxRange r("coupled");
       EHD_LAUNCH(s, 3, launch_coupled(s->kp, s->b, s->cur, s->stream));
     }

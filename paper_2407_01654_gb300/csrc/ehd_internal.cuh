@@ -310,7 +310,7 @@ struct Ctl {
   int redo;                 // streaming, several sub-iterations a launch: > 0: the rule stopped
                             // the loop inside the last launch; the next one repeats that many
                             // (one-cluster loop: > 0: a CTA of this solve gave up waiting)
-  int plaunch;              // streaming: launches of the current solve
+  int plaunch;              // and its launches in the current solve
   int guess;                // several sub-iterations a launch: those of the last solve (0: not known)
   unsigned oob;             // checked build: out-of-range indices met (see EHD_IDX)
 };

@@ -641,7 +641,7 @@ __device__ __forceinline__ void coupled_record(const KParams& k, StepState* ss, 
   d.sum_phi = sum_phi;
   d.sum_q = sum_q;
   d.barrier_error |= bar_error;
-  d.plaunches += plaunch;
+  d.plaunches += plaunch > 0 ? plaunch : it;  // (k_poisson makes one a launch and counts none)
   d.steps += 1;
   *stats = d;
   // values of the next step, in the other slot (this step's slot is being read)

@@ -193,7 +193,6 @@ __global__ void __launch_bounds__(THREADS, 8) k_poisson(KParams k, float* __rest
     }
     ctl->converged = conv;
     ctl->done = done;
-    ctl->plaunch = it;
     ctl->ticket_p = 0u;
     __threadfence();
     // inside a step graph: the while node repeats this kernel until the loop is done
