@@ -456,25 +456,33 @@ void first_form(ehd_sim* s) {
   s->h_ctl[1].iter = 0;
 }
 
-// After `steps` steps run as graphs: every 256 steps the device is asked for the count of its
-// last solve, the answer read 256 steps (or more, where the host runs ahead) later, so that
-// nothing waits.  Two answers in a row that ask for the other loop change over to it; the
-// states and decisions of the two are the same bit for bit.
+// Changes over to the form that solves of k sub-iterations ask for.
+void choose_form(ehd_sim* s, int k) {
+  s->want_one = one_step_wins(s, k);
+  if (s->want_one == s->one_step) return;
+  swap_forms(s);
+  ensure_graphs(s);
+  if (!s->graphs_ok) {
+    swap_forms(s);
+    s->two_forms = false;
+  }
+}
+
+// After `steps` steps run as graphs: every 128 steps the device is asked for the count of its
+// last solve, the answer read 128 steps (or more, where the host runs ahead) later, so that
+// nothing waits.  Two answers in a row that ask for the other form change over to it, as do
+// statistics of 64 steps or more that all took one count (fill_stats); the states and decisions
+// of the two are the same bit for bit.
 int follow_count(ehd_sim* s, int steps) {
-  constexpr int EVERY = 256;
+  constexpr int EVERY = 128;
   if (!s->two_forms || (s->form_steps += steps) < EVERY) return EHD_OK;
   s->form_steps = 0;
   const int k = *static_cast<volatile int*>(&s->h_ctl[1].iter);
-  const bool want_one = one_step_wins(s, k);
-  if (want_one == s->want_one && want_one != s->one_step) {
-    swap_forms(s);
-    ensure_graphs(s);
-    if (!s->graphs_ok) {
-      swap_forms(s);
-      s->two_forms = false;
-    }
+  if (k > 0) {  // 0: no answer yet
+    const bool want_one = one_step_wins(s, k);
+    if (want_one == s->want_one) choose_form(s, k);
+    s->want_one = want_one;
   }
-  s->want_one = want_one;
   EHD_CUDA(cudaMemcpyAsync(&s->h_ctl[1].iter, &s->b.ctl->iter, sizeof(int),
                            cudaMemcpyDeviceToHost, s->stream));
   return EHD_OK;
@@ -955,6 +963,10 @@ static int fill_stats(ehd_sim* s, ehd_stats* out) {
   out->last_rel_change = d.last_rel;
   out->sum_phi = d.sum_phi;
   out->sum_q = d.sum_q;
+  if (s->two_forms && s->graphs_ok && d.steps >= 64 && d.iters_min == d.iters_max) {
+    s->h_ctl[1].iter = d.iters_max;  // (the stream is idle: no older answer is on its way)
+    choose_form(s, d.iters_max);
+  }
   // host-driven launches are counted as they are queued; a graph step launches moments,
   // the potential loop (one resident kernel, or one kernel per sub-iteration) and coupled
   out->kernel_launches = s->launches + 2LL * s->graph_steps;

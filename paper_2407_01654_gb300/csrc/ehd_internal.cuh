@@ -311,7 +311,7 @@ struct Ctl {
                             // the loop inside the last launch; the next one repeats that many
                             // (one-cluster loop: > 0: a CTA of this solve gave up waiting)
   int plaunch;              // and its launches in the current solve
-  int guess;                // several sub-iterations a launch: those of the last solve (0: not known)
+  int guess, above;         // the count its launches aim at (0: not known); solves in a row past it
   unsigned oob;             // checked build: out-of-range indices met (see EHD_IDX)
 };
 

@@ -19,7 +19,7 @@
 // where FP64 sums in another order do.  The last CTA applies the rule to the n sub-iterations in
 // order.  When it stops the loop before the n-th, the state in the other copy of h, from which
 // this launch began, is advanced again by that many: one more launch per solve at most.  So that
-// settled solves need none, a launch aims at the count that the solve before took (multi_steps):
+// settled solves need none, a launch aims at the count that the solves before took (multi_steps):
 // with launches of five whatever the count a step took 371, 390, 408, 425 and 325 us at K = 1 ... 5
 // and 1024 x 2048, with these it takes 242, 265, 288, 300 and 325, with one sub-iteration a
 // launch 237, 296, 355, 414 and 473.
@@ -56,9 +56,9 @@ __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
 }
 
 // Sub-iterations the next launch makes.  A fixed count: what is left of it in equal launches.
-// Under the rule: the same up to the count of the solve before (`guess`, 0: not known), which the
-// next solve mostly takes again, so that the launch that ends it ends where the rule does; past
-// it one, two, four and then all that a launch may make.
+// Under the rule: the same up to the count that the solves before took (`guess`, 0: not known), so
+// that the launch that ends the solve mostly ends where the rule does; past it one, two, four and
+// then all that a launch may make.
 __device__ inline int multi_steps(int d, int fixed, int max_iter, int iter, int guess) {
   const int left = (fixed > 0 ? fixed : max_iter) - iter;
   int aim = left;
@@ -416,7 +416,16 @@ __global__ void __launch_bounds__(MT, 2)
       ctl->rel = rel;
       ctl->converged = conv;
     }
-    if (done) ctl->guess = iter + stop;
+    if (done) {
+      // A launch too many repeats a whole one, a launch too short costs one more of a single
+      // sub-iteration, a third of that: the guess falls at once, and rises when eight solves in
+      // a row went past it (counts of 4 and 5 in turn at 900 x 900: 184 us a step with the last
+      // count as the guess, 177 with launches of five).
+      const int k = iter + stop, guess = ctl->guess;
+      const int above = guess > 0 && k > guess ? ctl->above + 1 : 0;
+      if (k < guess || guess <= 0 || above >= 8) ctl->guess = k;
+      ctl->above = above >= 8 ? 0 : above;
+    }
     if (done && stop < n) {
       ctl->redo = stop;  // the next launch repeats this one's first sub-iterations
       done = 0;

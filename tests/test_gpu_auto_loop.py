@@ -60,9 +60,11 @@ def test_settled_counts_choose_the_loop(gpu, nx, ny, precision, k, settled):
         s.set_fields(*f)
         stays = {1: first}.get(over.get("poisson_loop"), over.get("poisson_loop"))
         assert loop_of(s) == (stays or first)
-        for n in (3, 600, 700, 257):  # calls that end between two looks at the count, and odd ones
+        for n in (3, 60, 61, 700, 257):  # calls that end between two looks at the count, and odd ones
             st = s.step(n)
             assert st["poisson_iters_min"] == st["poisson_iters_max"] == k and st["steps"] == n
+            if n < 64:  # neither a look's answer nor enough steps of one count
+                assert loop_of(s) == (stays or first)
         assert loop_of(s) == (stays or settled)
         ends.append(s.read_fields())
         blob = s.save_state()
@@ -70,8 +72,7 @@ def test_settled_counts_choose_the_loop(gpu, nx, ny, precision, k, settled):
             for again in (lambda: s.set_fields(*f), lambda: s.load_state(blob)):
                 again()
                 assert loop_of(s) == first
-                for n in (1200, 300, 300):  # (the host runs ahead of the device inside a call)
-                    s.step(n)
+                s.step(64)  # as many of one count as its statistics need to tell
                 assert loop_of(s) == settled
         s.close()
     for name in ends[0]:
@@ -95,7 +96,7 @@ def test_single_steps_and_profiling(gpu):
     p, f = setup(300, 300, 1)
     s = gpu.Sim(p)
     s.set_fields(*f)
-    for _ in range(1100):
+    for _ in range(600):
         s.step(1)
     assert s.loop_kind() == 2
     s.profile(True)
@@ -106,8 +107,23 @@ def test_single_steps_and_profiling(gpu):
     s.close()
     s = gpu.Sim(dict(p, poisson_loop=3))
     s.set_fields(*f)
-    s.step(1104)
+    s.step(604)
     b = s.read_fields()
     s.close()
     for name in a:
         assert np.array_equal(a[name], b[name]), name
+
+
+def test_calls_without_statistics_follow_the_count(gpu):
+    """Nothing is read back but the count; the answers of a long call arrive while it is queued or
+    before the next one."""
+    p, f = setup(300, 300, 1)
+    s = gpu.Sim(p)
+    s.set_fields(*f)
+    for _ in range(4):
+        s.step(200, stats=False)
+        s.read_fields(("phi",))
+    assert s.loop_kind() == 2
+    st = s.read_stats()
+    assert st["steps"] == 800 and st["poisson_iters_total"] == 800
+    s.close()
