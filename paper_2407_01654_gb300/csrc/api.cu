@@ -937,7 +937,8 @@ int ehd_set_fields(ehd_sim* s, const void* phi, const void* q, const void* ux, c
   // the populations are written into the current copy; the potential restarts in copy 0
   EHD_CUDA(cudaMemsetAsync(&s->b.ctl->parity, 0, sizeof(int), s->stream));
   EHD_CUDA(cudaMemsetAsync(&s->b.ctl->nonfinite, 0, sizeof(int), s->stream));
-  if (s->multi) EHD_CUDA(cudaMemsetAsync(&s->b.ctl->guess, 0, sizeof(int), s->stream));
+  // (the count that the streaming launches aim at: of other fields it says nothing)
+  if (s->multi) EHD_CUDA(cudaMemsetAsync(&s->b.ctl->guess, 0, 3 * sizeof(int), s->stream));
   s->launches += 1;
   EHD_CUDA(launch_step_set(s->kp, s->b, s->cur, s->n, 1, s->stream));
   EHD_LAUNCH(s, 0, launch_init(s->kp, s->b, s->cur, p != nullptr, s->stream));

@@ -312,6 +312,7 @@ struct Ctl {
                             // (one-cluster loop: > 0: a CTA of this solve gave up waiting)
   int plaunch;              // and its launches in the current solve
   int guess, above;         // the count its launches aim at (0: not known); solves in a row past it
+  int aim;                  // and what the next launch may make under the rule (0: all)
   unsigned oob;             // checked build: out-of-range indices met (see EHD_IDX)
 };
 

@@ -19,7 +19,7 @@
 // where FP64 sums in another order do.  The last CTA applies the rule to the n sub-iterations in
 // order.  When it stops the loop before the n-th, the state in the other copy of h, from which
 // this launch began, is advanced again by that many: one more launch per solve at most.  So that
-// settled solves need none, a launch aims at the count that the solves before took (multi_steps):
+// settled solves need none, a launch aims at the count that the solves before took (multi_aim):
 // with launches of five whatever the count a step took 371, 390, 408, 425 and 325 us at K = 1 ... 5
 // and 1024 x 2048, with these it takes 242, 265, 288, 300 and 325, with one sub-iteration a
 // launch 237, 296, 355, 414 and 473.
@@ -55,22 +55,41 @@ __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
                : "memory");
 }
 
-// Sub-iterations the next launch makes.  A fixed count: what is left of it in equal launches.
-// Under the rule: the same up to the count that the solves before took (`guess`, 0: not known), so
-// that the launch that ends the solve mostly ends where the rule does; past it one, two, four and
-// then all that a launch may make.
-__device__ inline int multi_steps(int d, int fixed, int max_iter, int iter, int guess) {
+// Sub-iterations the next launch may make: what is left of a fixed count in equal launches, or
+// under the rule as many as it may.
+__host__ __device__ inline int multi_steps(int d, int fixed, int max_iter, int iter) {
   const int left = (fixed > 0 ? fixed : max_iter) - iter;
-  int aim = left;
-  if (fixed <= 0) {
-    if (guess <= 0) return left < d ? left : d;
-    const int past = iter - guess;
-    aim = past < 0 ? -past : (past + 1 < d ? past + 1 : d);
-    if (aim > left) aim = left;
-  }
+  if (left <= d) return left;
+  if (fixed <= 0) return d;
+  const int launches = (left + d - 1) / d;
+  return (left + launches - 1) / launches;
+}
+// Under the rule, after `iter` sub-iterations: equal launches up to the count that the solves before
+// took (`guess`, 0: not known), so that the launch that ends the solve mostly ends where the
+// rule does; past it one, two, four and then all that a launch may make.
+__device__ inline int multi_aim(int d, int guess, int iter) {
+  if (guess <= 0) return d;
+  const int past = iter - guess;
+  const int aim = past < 0 ? -past : (past + 1 < d ? past + 1 : d);
   if (aim <= d) return aim;
   const int launches = (aim + d - 1) / d;
   return (aim + launches - 1) / launches;
+}
+
+// Keeps the aim of the next launch after k sub-iterations of a solve under the rule.
+// A launch too many repeats a whole one, a launch too short costs one more of a single
+// sub-iteration, a third of that: the guess falls at once, and rises when eight solves in a row
+// went past it (counts of 4 and 5 in turn at 900 x 900: 184 us a step with the last count as the
+// guess, 177 with launches of five, 177 so).
+// (Out of line: in line it moved the loops above it, 63.7 us a solve at 977 x 811 against 62.8.)
+__device__ __noinline__ void keep_aim(Ctl* ctl, int d, int k, int done) {
+  int guess = ctl->guess;
+  if (done) {
+    const int above = guess > 0 && k > guess ? ctl->above + 1 : 0;
+    if (k < guess || guess <= 0 || above >= 8) ctl->guess = guess = k;
+    ctl->above = above >= 8 ? 0 : above;
+  }
+  ctl->aim = multi_aim(d, guess, done ? 0 : k);
 }
 
 }  // namespace
@@ -96,8 +115,9 @@ __global__ void __launch_bounds__(MT, 2)
   const bool bad_state = __ldg(&ctl->nonfinite) != 0;
   const int fixed = bad_state ? 0 : __ldg(&ctl->fixed_iter),
             max_iter = bad_state ? 1 : __ldg(&ctl->max_iter);
-  const int iter = __ldg(&ctl->iter), redo = __ldg(&ctl->redo);
-  const int n = redo > 0 ? redo : multi_steps(D, fixed, max_iter, iter, __ldg(&ctl->guess));
+  const int iter = __ldg(&ctl->iter), redo = __ldg(&ctl->redo), aim = __ldg(&ctl->aim);
+  int n = redo > 0 ? redo : multi_steps(D, fixed, max_iter, iter);
+  if (fixed <= 0 && redo == 0 && aim > 0 && aim < n) n = aim;
   const int nx = k.nx, ny = k.ny;
   const size_t N = (size_t)k.N;
   const float* __restrict__ src = hbuf + (size_t)parity * NH * N;
@@ -416,16 +436,7 @@ __global__ void __launch_bounds__(MT, 2)
       ctl->rel = rel;
       ctl->converged = conv;
     }
-    if (done) {
-      // A launch too many repeats a whole one, a launch too short costs one more of a single
-      // sub-iteration, a third of that: the guess falls at once, and rises when eight solves in
-      // a row went past it (counts of 4 and 5 in turn at 900 x 900: 184 us a step with the last
-      // count as the guess, 177 with launches of five).
-      const int k = iter + stop, guess = ctl->guess;
-      const int above = guess > 0 && k > guess ? ctl->above + 1 : 0;
-      if (k < guess || guess <= 0 || above >= 8) ctl->guess = k;
-      ctl->above = above >= 8 ? 0 : above;
-    }
+    if (fixed <= 0 && !bad_state) keep_aim(ctl, D, iter + stop, done);
     if (done && stop < n) {
       ctl->redo = stop;  // the next launch repeats this one's first sub-iterations
       done = 0;
